@@ -283,7 +283,7 @@ __device__ __forceinline__ int ceil_log2_u32(uint32_t m) { return m <= 1u ? 0 : 
 // (literal as long as the levels before were right).  A slice outside the
 // BF16 range (or a non-finite input) anywhere in the operand sends every
 // vector to the literal passes, which flag such slices as Eq. (fp64split)
-// computes them.
+// computes them.  ff may be the first row of vmax.
 __device__ __forceinline__ void rc_verify_pass(const uint32_t *vmax, int32_t *vrc, int32_t *ff, int64_t nvec,
                                                WsHeader *ws, int slot, int64_t tid, int64_t nthreads)
 {
@@ -386,10 +386,13 @@ cudaError_t launch_split_f64_rc(const double *X, int64_t rows, int64_t cols, int
 {
     const int64_t nvec = transpose ? cols : rows;
     const int64_t plane = nvec * ldcomp;
-    // scratch: literal maxima [nvec] u64, speculative maxima [5][nvec] u32, ff [nvec] i32
+    // scratch (rc_scratch_bytes): literal maxima [nvec] u64, speculative maxima [5][nvec]
+    // u32.  ff [nvec] i32 takes the place of the first row of the speculative
+    // maxima: the verifier's thread reads a vector's five maxima before it
+    // writes the vector's ff, and nothing reads them after that.
     auto *maxbits = static_cast<unsigned long long *>(scratch);
     auto *vmax = reinterpret_cast<uint32_t *>(maxbits + nvec);
-    int32_t *ff = reinterpret_cast<int32_t *>(vmax + 5 * nvec);
+    int32_t *ff = reinterpret_cast<int32_t *>(vmax);
     if (nvec == 0) return cudaSuccess;
     const int lgrid = grid_for((nvec + 255) / 256, 152 * 4);
     cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)nvec * (8 + 20), st);
