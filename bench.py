@@ -224,10 +224,9 @@ class Case:
             self.gemm_ws = emu.workspace(emu.emu_gemm_f64_merged_workspace_bytes(M, N, K), dev)
         if self.api:
             self.gemm_ws = emu.workspace(emu.emu_gemm_workspace_bytes(self.mode, M, N, K), dev)
-        # the product-sum kernel that runs: FP64 mode has 128 x 128 tiles and 256-column tiles
-        # (128 x 256 on one SM, 256 x 256 on a pair of SMs), both kernels named after their file
-        self.kernel = "prodsum_f32" if self.mode == 32 else \
-            "prodsum_f64w" if emu.emu_prodsum_f64_tile_columns(M, N) == 256 else "prodsum_f64"
+        # the product-sum kernel that runs, named after its file (FP64: one kernel for every tile
+        # shape; prodsum_f64n.cu compiles its narrower tiles)
+        self.kernel = "prodsum_f32" if self.mode == 32 else "prodsum_f64w"
         # the kernel's own name (FP32: 256 x 256 tiles on CTA pairs have a kernel of their own)
         self.kernel_name = "prodsum_f32_pair_kernel" if self.mode == 32 and emu.emu_prodsum_f32_tile_rows(M, N) == 256 \
             else self.kernel + "_kernel"
@@ -235,7 +234,7 @@ class Case:
         self.exec_flop = self.flop * (6 if self.mode == 32 else self.nprod)
         # kernels of ours per step: FP32 split of both operands = 1 launch; FP64 split of both =
         # 5 (level maxima of both, then a speculative pass and a verifier per operand);
-        # product-sum = 1, or 2 when the library runs the last partial wave of 256-column
+        # product-sum = 1, or 2 when the library runs the last partial wave of its widest
         # tiles as 128 x 128 tiles (it reports its schedule)
         self.launches = 1 if self.fused else 1 + emu.emu_prodsum_f32_launches(M, N) if self.mode == 32 else \
             5 + emu.emu_prodsum_f64_launches(M, N)

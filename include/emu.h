@@ -204,8 +204,9 @@ emu_status emu_gemm_f32_fused(int64_t M, int64_t N, int64_t K, const float *A, i
  * each, the FP32 component product fl32(A_i B_j) is formed on the tensor
  * cores per K-chunk of 256 (every chunk partial is exact, Section 5.2), the
  * partials are summed exactly, and the total is added once into the FP64
- * result: C <- fl64(C + fl32(A_i B_j)).  C equals the oracle's product-outer
- * order bit for bit.  The FP64 accumulator lives in the workspace; C serves
+ * result: C <- fl64(C + fl32(A_i B_j)) (products of a diagonal may be added
+ * together where that gives the same bits).  C equals the oracle's
+ * product-outer order bit for bit.  The FP64 accumulator lives in the workspace; C serves
  * as scratch for low-order words of the exact sums while the kernel runs. */
 emu_status emu_gemm_f64(int64_t M, int64_t N, int64_t K, const double *A, int64_t lda,
                         const double *B, int64_t ldb, double *C, int64_t ldc, int nprod,
@@ -319,10 +320,10 @@ int emu_prodsum_f32_tile_rows(int64_t M, int64_t N);
 int emu_prodsum_f32_launches(int64_t M, int64_t N);
 
 /* Output-tile shape that the FP64-mode product-sum picks for an M x N
- * result, unless EMU_F64_TILE (128x128, 128x256 or 256x256) forces one:
- * width 128 or 256 columns; height 128 rows, or 256 rows where a 256-column
+ * result, unless EMU_F64_TILE (128x64, 128x128, 128x256 or 256x256) forces one:
+ * width 64, 128 or 256 columns; height 128 rows, or 256 rows where a 256-column
  * tile runs on a pair of SMs (a cluster of two CTAs sharing each MMA); and
- * the number of kernel launches (2 when the last, partial wave of 256-column
+ * the number of kernel launches (2 when the last, partial wave of 256-row
  * tiles runs as 128 x 128 tiles in a second launch).  The paper has no
  * counterpart: every shape gives identical results, and the calls only
  * report which kernels run.  0 for sizes < 1. */
