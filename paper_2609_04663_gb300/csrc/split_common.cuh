@@ -469,10 +469,11 @@ f64_max_kernel(const double *__restrict__ X, int64_t rows, int64_t cols, int64_t
 }
 
 // One thread: checks the speculative levels in order.  Level r's max from
-// the fused pass is literal as long as levels < r were right and it spans
-// at least two units 2^(v0 - 50) of the fixed point (below that the sticky
-// bit of the truncated residual decides its power of two), so the first
-// mismatch r gives the true v^(r) directly when v^(r) >= v0 - 48 and levels
+// the fused pass gives the literal v^(r) as long as levels < r were right and
+// it spans at least one of the units it is kept in (2^(v0 - 22) for level 1,
+// 2^(v0 - 37) for levels 2 and 3), or two units 2^(v0 - 50) of the fixed point
+// (below that the sticky bit of the truncated residual decides its power of
+// two), so the first mismatch r gives the true v^(r) directly then and levels
 // after r are redone; a smaller one is redone from level r itself.  A
 // slice outside the BF16 normal range at level r (a domain violation, which
 // the finalizer flags) also ends the trusted levels at r: the fused pass
@@ -501,7 +502,7 @@ __device__ __forceinline__ int f64_verify_levels(const WsHeader *ws, int slot, i
             const int vr = ceil_log2_bits(m);
             v[r] = vr;
             if (r == badlvl) ff = r;
-            else if (vr != v0 - 8 * r) ff = vr >= v0 - 48 ? r : r - 1;
+            else if (vr != v0 - 8 * r) ff = vr >= v0 - (r == 1 ? 22 : r <= 3 ? 37 : 48) ? r : r - 1;
         }
     }
     return ff;
@@ -555,163 +556,135 @@ __device__ __forceinline__ void grid_sync(WsHeader *ws, int slot)
 }
 
 // ------------------------------------------ FP64 speculative pass kernels
-// The levels of spec_levels restated so that most steps are 32-bit: levels 0
-// and 1 have grids of 2^32 units or coarser and round on the upper word of
-// the fixed-point magnitude (the lower word only breaks ties and is carried
-// into the residual), level 2 rounds a value below 2^35 through its quotient
-// and remainder, and levels 3-5 work in 32 bits.  At each level the grid
-// splits |X| into t = |X| >> g and a remainder; rounding up (remainder above
-// half the grid, or exactly half with t odd) leaves the grid minus the
-// remainder with the opposite sign.  No range check is needed when
-// v0 >= -78: every nonzero slice then lies between 2^(v0 - 48) >= 2^-126 and
-// 2^v0 <= 2^127.  Results are bit-identical to spec_levels.
-// Slices are returned as 32-bit words holding the FP32 value of the slice,
-// whose upper 16 bits are its BF16 bits (the value has at most 8 significant
-// bits, so the lower 16 are zero); two words pack into one plane word with a
-// byte permutation.  The arithmetic runs on the FP32 pipe: n (an integer
-// <= 256) is converted exactly (2^23 + n by bits, minus 2^23) and scaled by
-// the level's unit, a power of two, with the sign of the residual (whose grid
-// is half as coarse when negative: -1/2).  All values are normal floats on
-// the fast path.  The FMA with +0 keeps a zero slice +0.
-__device__ __forceinline__ uint32_t slice_word(uint32_t n, uint32_t sg, float unit)
+// The levels of spec_levels restated in FP32 arithmetic, where an entry's
+// levels take a handful of instructions each (the pass is bound by
+// instruction issue, not by memory; GB300's FP64 pipe is far too slow for the
+// literal add-subtract form).  The fixed-point magnitude X (units of 2^F, F = v0 -
+// 50, below 2^50 + 1, truncated bits jammed into the last one) is cut into
+// pieces that FP32 holds exactly, two levels to a piece:
+// - levels 0, 1: Xh = X >> 28 (at most 2^22) plus 1/2 if the 28 bits below are
+//   not all zero.  Grids and half-grids are integers in these units, so the 1/2
+//   breaks exactly the ties the bits below break, in their direction, and
+//   compares with powers of two as the exact value does;
+// - levels 2, 3: the residual (an integer of at most 2^7) rejoined with the 28
+//   bits, again without its lowest 13 bits and plus 1/2 for them (two's
+//   complement: they count upwards);
+// - levels 4, 5: what is left, below 2^19, exactly.
+// Each level is the projection's own add-subtract with C = 1.5 * 2^23 grids,
+// which rounds to nearest, ties to even, on the grid 2^(43 - 8r) units for a
+// non-negative residual and half of it for a negative one (the sign-dependent
+// grid of Eq. (fp64split)).  Slices are returned as 32-bit words holding the
+// FP32 value of the slice, whose upper 16 bits are its BF16 bits (at most 8
+// significant bits, so the lower 16 are zero); two words pack into one plane
+// word with a byte permutation.  No range check is needed when v0 >= -78: every
+// nonzero slice then lies between 2^(v0 - 48) >= 2^-126 and 2^v0.  Slices are
+// bit-identical to spec_levels.  About 120 instructions an entry with six
+// slices (150 in the transposed pass; 193 and 218 with the levels in 32- and
+// 64-bit integers): 4096 x 4096 rows 106 -> 78 us, transposed 114 -> 83 us.
+// The maxima |X^(r)| before levels 1 .. 5 are in units of 2^(F + kMagShift[r - 1]),
+// rounded to an odd half as above: they decide comparisons with powers of two
+// of at least one unit.
+__device__ constexpr int kMagShift[5] = {28, 13, 13, 0, 0};
+
+// Scales of the pieces: units of 2^(F + 28), 2^(F + 13) and 2^F in value (the
+// last is a subnormal number for v0 < -76; multiplying by it is exact).
+__device__ __forceinline__ void spec_units(int F, float (&P)[3])
 {
-    const float fn = __fsub_rn(__uint_as_float(0x4B000000u + n), 8388608.0f);
-    const float us = __fmul_rn(unit, __uint_as_float(0x3F800000u + sg * 0x7F800000u));   // +1 or -1/2
-    return __float_as_uint(__fmaf_rn(fn, us, 0.0f));
+    P[0] = __int_as_float((F + 28 + 127) << 23);
+    P[1] = __fmul_rn(P[0], 0x1p-15f);
+    P[2] = __fmul_rn(P[0], 0x1p-28f);
 }
 
-// Slice word of an FP32 value z (a multiple of the level's grid 2^c or 2^(c-1)
-// units, at most nine significant bits) in units of 2^F: z * 2^-c * 2^(F + c),
-// both steps exact; a zero z gives +0.
-__device__ __forceinline__ uint32_t slice_word_scaled(float z, float inv_grid, float unit)
+// One level on a piece: the slice's word, y <- y - z.  grid: the level's grid
+// for y >= 0 in y's units.
+__device__ __forceinline__ uint32_t piece_level(float &y, float grid, float unit)
 {
-    return __float_as_uint(__fmul_rn(__fmul_rn(z, inv_grid), unit));
-}
-
-// Units of the six levels of the fast path: 2^(F + 43 - 8r), r = 0..5 (the
-// grid of a non-negative residual at level r, in value).
-__device__ __forceinline__ void spec_units(int F, float (&P)[6])
-{
-    P[0] = __int_as_float((F + 43 + 127) << 23);
-#pragma unroll
-    for (int r = 1; r < 6; ++r) P[r] = __fmul_rn(P[r - 1], 0.00390625f);          // 2^-8
+    const float C = (y < 0.0f) ? 6291456.0f * grid : 12582912.0f * grid;      // 1.5 * 2^22, 1.5 * 2^23
+    const float z = __fsub_rn(__fadd_rn(y, C), C);
+    y = __fsub_rn(y, z);
+    return __float_as_uint(__fmul_rn(z, unit));
 }
 
 template <int NLEV>
-__device__ __forceinline__ void spec_levels_fast(double x, int F, const float (&P)[6], uint32_t (&s)[6],
-                                                 uint32_t &badmask, unsigned long long &m1, unsigned long long &m2,
-                                                 uint32_t (&m)[3])
+__device__ __forceinline__ void spec_levels_fast(double x, int v0, const float (&P)[3], uint32_t (&s)[6],
+                                                 uint32_t &badmask, float (&m)[5])
 {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    uint32_t sg = (uint32_t)(b >> 63);
-    const int E = (int)((b >> 52) & 0x7FFu);
-    uint64_t M = b & 0x000FFFFFFFFFFFFFull;
-    int Ee = E;
-    if (E == 0) Ee = 1; else M |= 1ull << 52;
-    if (E == 0x7FF) { badmask |= 1u; M = 0; }          // a non-finite slice 0
-    const int sh0 = (Ee - 1075) - F;
-    uint64_t a;
-    if (M == 0) a = 0;
-    else if (sh0 >= 0) a = sh0 < 12 ? (M << sh0) : (1ull << 62);
-    else if (sh0 > -64) a = (M >> (-sh0)) | ((M << (64 + sh0)) != 0 ? 1ull : 0ull);
-    else a = 1;
-    uint32_t H = (uint32_t)(a >> 32), L = (uint32_t)a;
-    // At every level the rounding is written as multiply-adds where it can
-    // be: with the grid 2^g (g one lower for a negative residual), t the
-    // truncated quotient, rem = X - t 2^g and b the bits below the grid word
-    // (a sticky bit for levels 0 and 1), rounding up happens exactly when
-    // 2 rem + b + (t & 1) > 2^g (above half, or a tie with t odd); then the new
-    // residual is 2^g - rem - b with the opposite sign.
-    // levels 0, 1: grid 2^(32 + gh) units, gh = 11 / 10 and 3 / 2
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        if (r == 1) {
-            const unsigned long long cur = ((unsigned long long)H << 32) | L;
-            m1 = cur > m1 ? cur : m1;
-        }
-        constexpr uint32_t kG[2] = {1u << 11, 1u << 3};
-        const uint32_t grid = kG[r] - sg * (kG[r] >> 1);
-        const uint32_t t = H >> ((11 - 8 * r) - (int)sg);
-        const uint32_t rh = H - t * grid;
-        const uint32_t lnz = min(L, 1u);
-        const uint32_t lsb = t & 1u;
-        const int32_t d = (int32_t)(grid - 2u * rh - lnz - lsb);
-        const uint32_t up = (uint32_t)d >> 31;
-        s[r] = slice_word(t + up, sg, P[r]);
-        H = rh + up * ((uint32_t)d + lsb);
-        L = L * (1u - 2u * up);
-        sg ^= up;
+    const uint32_t xh = (uint32_t)__double2hiint(x), ml = (uint32_t)__double2loint(x);
+    const uint32_t E = (xh >> 20) & 0x7FFu, sign = xh & 0x80000000u;
+    if (E == 0x7FFu) badmask |= 1u;                    // a non-finite slice 0 (its planes are unspecified)
+    const uint32_t mh = (xh & 0xFFFFFu) | (E ? 0x100000u : 0u);
+    // U = significand * 2^10 (uh:ul); |x| = (U >> t) units of 2^(v0 - 62), t >= 0
+    const uint32_t uh = __funnelshift_l(ml, mh, 10), ul = ml << 10;
+    const int t = v0 + 1023 - (int)E;
+    const uint32_t Xh = __funnelshift_rc(uh, 0u, (uint32_t)(t + 8));           // U >> (t + 40)
+    uint32_t w, drop;                                  // low word of U >> (t + 12); what that drops
+    if ((uint32_t)t < 20u) {
+        w = __funnelshift_r(ul, uh, t + 12);
+        drop = ml << (30 - t);
+    } else {
+        w = __funnelshift_rc(uh, 0u, (uint32_t)(t - 20));
+        drop = t <= 30 ? ml << (30 - t) : (ml | (mh << (t < 62 ? 62 - t : 0)));
+        if (t < 0) w = drop = 0;                       // not finite, or above 2^v0: cannot occur in the domain
     }
-    // level 2: |X| < 2^35, grid 2^27 / 2^26
-    uint32_t Y;
-    {
-        const unsigned long long cur = ((unsigned long long)H << 32) | L;
-        m2 = cur > m2 ? cur : m2;
-        const uint32_t grid = (1u << 27) - sg * (1u << 26);
-        const uint32_t t = __funnelshift_r(L, H, 27 - (int)sg);
-        const uint32_t rem = L - t * grid;
-        const uint32_t lsb = t & 1u;
-        const int32_t d = (int32_t)(grid - 2u * rem - lsb);
-        const uint32_t up = (uint32_t)d >> 31;
-        s[2] = slice_word(t + up, sg, P[2]);
-        Y = rem + up * ((uint32_t)d + lsb);
-        sg ^= up;
-    }
+    const uint32_t Xl = (w & 0x0FFFFFFFu) | min(drop, 1u);
+    // levels 0, 1
+    float y = __fsub_rn(__uint_as_float(0x4B000000u | Xh), Xl ? 8388607.5f : 8388608.0f);
+    y = __uint_as_float(__float_as_uint(y) ^ sign);
+    s[0] = piece_level(y, 0x1p15f, P[0]);
+    m[0] = fmaxf(m[0], fabsf(y));
+    s[1] = piece_level(y, 0x1p7f, P[0]);
+    // levels 2, 3: y without its half is the integer r; (r 2^28 + sX) >> 13 and the 13 bits below
+    const int32_t sX = sign ? -(int32_t)Xl : (int32_t)Xl;
+    const float r = __fsub_rn(y, Xl ? __uint_as_float(0x3F000000u | sign) : 0.0f);
+    const uint32_t rb = __float_as_uint(__fadd_rn(r, 12582912.0f));              // 0x4B400000 + r
+    const uint32_t yb = (rb << 15) + (uint32_t)(sX >> 13) + (0x4B400000u - (0x4B400000u << 15));
+    const uint32_t Yl = (uint32_t)sX & 0x1FFFu;
+    const float p = Yl ? 0.5f : 0.0f;
+    y = __fadd_rn(__fsub_rn(__uint_as_float(yb), 12582912.0f), p);
+    m[1] = fmaxf(m[1], fabsf(y));
+    s[2] = piece_level(y, 0x1p14f, P[1]);
     if constexpr (NLEV <= 3) return;                   // levels from NLEV on are not wanted
-    // level 3: |X| <= 2^26, grid 2^19 / 2^18
-    {
-        m[0] = Y > m[0] ? Y : m[0];
-        const uint32_t grid = (1u << 19) - sg * (1u << 18);
-        const uint32_t t = Y >> (19 - (int)sg);
-        const uint32_t rem = Y - t * grid;
-        const uint32_t lsb = t & 1u;
-        const int32_t d = (int32_t)(grid - 2u * rem - lsb);
-        const uint32_t up = (uint32_t)d >> 31;
-        s[3] = slice_word(t + up, sg, P[3]);
-        Y = rem + up * ((uint32_t)d + lsb);
-        sg ^= up;
-    }
+    m[2] = fmaxf(m[2], fabsf(y));
+    s[3] = piece_level(y, 0x1p6f, P[1]);
     if constexpr (NLEV <= 4) return;
-    // levels 4, 5: |X| <= 2^18, exact in FP32; the add-subtract projection
-    // with C = 1.5 * 2^(23 + g) rounds to the grid 2^g to nearest, ties to even
-    float y = __fsub_rn(__uint_as_float(0x4B000000u | Y), 8388608.0f);
-    y = sg ? -y : y;
-#pragma unroll
-    for (int r = 4; r < 6; ++r) {
-        if (r >= NLEV) break;
-        const float ay = fabsf(y);
-        m[r - 3] = max(m[r - 3], (uint32_t)ay);                   // exact: an integer below 2^24
-        const float C = (y < 0.0f) ? (r == 4 ? 12884901888.0f : 50331648.0f)      // 1.5 * 2^33, 1.5 * 2^25
-                                   : (r == 4 ? 25769803776.0f : 100663296.0f);    // 1.5 * 2^34, 1.5 * 2^26
-        const float z = __fsub_rn(__fadd_rn(y, C), C);
-        s[r] = slice_word_scaled(z, r == 4 ? 0.00048828125f : 0.125f, P[r]);     // 2^-11, 2^-3
-        y = __fsub_rn(y, z);
-    }
+    // levels 4, 5
+    y = __fmaf_rn(__fsub_rn(y, p), 8192.0f, __fsub_rn(__uint_as_float(0x4B000000u | Yl), 8388608.0f));
+    m[3] = fmaxf(m[3], fabsf(y));
+    s[4] = piece_level(y, 0x1p11f, P[2]);
+    if constexpr (NLEV <= 5) return;
+    m[4] = fmaxf(m[4], fabsf(y));
+    s[5] = piece_level(y, 0x1p3f, P[2]);
 }
 
-// Per-thread state of the speculative pass: level maxima in units of 2^F.
+// Per-thread state of the speculative pass: level maxima (kMagShift units).
 struct SpecState {
-    unsigned long long m1 = 0, m2 = 0;
-    uint32_t m[3] = {0, 0, 0};
+    float m[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     uint32_t badmask = 0;
 };
 
+// A magnitude in units of 2^F as the fast path would give it.
+__device__ __forceinline__ float mag_float(unsigned long long mx, int shift)
+{
+    const uint32_t q = (uint32_t)(mx >> shift);
+    return __fadd_rn((float)q, (mx & ((1ull << shift) - 1ull)) ? 0.5f : 0.0f);
+}
+
 // Slices 0 .. NLEV-1 of one entry (NLEV = 3..6; later ones are not formed).
 template <int NLEV = 6>
-__device__ __forceinline__ void spec_element(double x, int v0, bool fast, const float (&P)[6], uint32_t (&s)[6],
+__device__ __forceinline__ void spec_element(double x, int v0, bool fast, const float (&P)[3], uint32_t (&s)[6],
                                              SpecState &st)
 {
     if (v0 == kZeroLevel) {
 #pragma unroll
         for (int r = 0; r < 6; ++r) s[r] = 0;
     } else if (fast) {
-        spec_levels_fast<NLEV>(x, v0 - 50, P, s, st.badmask, st.m1, st.m2, st.m);
+        spec_levels_fast<NLEV>(x, v0, P, s, st.badmask, st.m);
     } else {                                          // tiny matrices: the checked general form
         uint16_t t[6];
-        unsigned long long mx[5] = {st.m1, st.m2, st.m[0], st.m[1], st.m[2]};
+        unsigned long long mx[5] = {0, 0, 0, 0, 0};
         spec_levels(x, v0, t, st.badmask, mx);
-        st.m1 = mx[0]; st.m2 = mx[1];
-        st.m[0] = (uint32_t)mx[2]; st.m[1] = (uint32_t)mx[3]; st.m[2] = (uint32_t)mx[4];
+#pragma unroll
+        for (int r = 0; r < 5; ++r) st.m[r] = fmaxf(st.m[r], mag_float(mx[r], kMagShift[r]));
 #pragma unroll
         for (int r = 0; r < 6; ++r) s[r] = (uint32_t)t[r] << 16;
     }
@@ -722,27 +695,26 @@ __device__ __forceinline__ uint32_t pack2(uint32_t lo, uint32_t hi) { return __b
 
 // Block-wide publication of the slice flags and the level maxima (as FP64
 // bit patterns of |A^(r)|, r = 1..5).  Every thread of the block calls it.
-__device__ __forceinline__ void spec_publish(const SpecState &st, int v0, WsHeader *ws, int slot, unsigned long long *red)
+__device__ __forceinline__ void spec_publish(const SpecState &st, int v0, WsHeader *ws, int slot, uint32_t *red)
 {
     const uint32_t bm = __reduce_or_sync(0xFFFFFFFFu, st.badmask);
     if (bm && lane_id() == 0) atomicOr(&ws->slice_bad[slot], bm);
-    // maxima in units (integers, so the reduction needs no conversion); one
-    // thread converts the block's five maxima to FP64 bit patterns
-    unsigned long long mm[5] = {st.m1, st.m2, st.m[0], st.m[1], st.m[2]};
+    // maxima as bits of non-negative floats, which order like them; one thread
+    // converts the block's five maxima to FP64 bit patterns
     const int w = threadIdx.x >> 5;
 #pragma unroll
     for (int r = 0; r < 5; ++r) {
-        mm[r] = warp_max(mm[r]);
-        if (lane_id() == 0) red[r * (kThreads / 32) + w] = mm[r];
+        const uint32_t mm = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(st.m[r]));
+        if (lane_id() == 0) red[r * (kThreads / 32) + w] = mm;
     }
     __syncthreads();
     if (threadIdx.x < 5) {
         const int r = threadIdx.x;
-        unsigned long long m = 0;
-        for (int i = 0; i < kThreads / 32; ++i) m = red[r * (kThreads / 32) + i] > m ? red[r * (kThreads / 32) + i] : m;
+        uint32_t m = 0;
+        for (int i = 0; i < kThreads / 32; ++i) m = max(m, red[r * (kThreads / 32) + i]);
         if (m) {
             const int F = (v0 == kZeroLevel) ? 0 : v0 - 50;
-            const double v = (double)m * pow2_d(F);                   // exact: below 2^53 units
+            const double v = (double)__uint_as_float(m) * pow2_d(F + kMagShift[r]);           // exact
             atomicMax(&ws->maxbits[slot][r + 1], (unsigned long long)__double_as_longlong(v));
         }
     }

@@ -32,11 +32,11 @@ template <int NLEV>
 __device__ __forceinline__ void f64_spec_rows_body(const double *__restrict__ X, int64_t rows, int64_t cols,
                                                    int64_t ldx, uint16_t *__restrict__ comps, int64_t ldcomp,
                                                    int64_t plane, WsHeader *ws, int slot, int64_t bx, int64_t by,
-                                                   int64_t gy, unsigned long long *red)
+                                                   int64_t gy, uint32_t *red)
 {
     const int v0 = spec_v0(ws, slot);
     const bool fast = v0 >= -78;
-    float P[6] = {};
+    float P[3] = {};
     if (fast) spec_units(v0 - 50, P);
     const bool vin = ((ldx & 1) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
     const bool vout = ((ldcomp & 3) == 0) && ((plane & 3) == 0) && ((reinterpret_cast<uintptr_t>(comps) & 7u) == 0);
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kThreads)
 f64_spec_rows_kernel(const double *__restrict__ X, int64_t rows, int64_t cols, int64_t ldx,
                      uint16_t *__restrict__ comps, int64_t ldcomp, int64_t plane, WsHeader *ws, int slot)
 {
-    __shared__ unsigned long long red[5 * (kThreads / 32)];
+    __shared__ uint32_t red[5 * (kThreads / 32)];
     f64_spec_rows_body<NLEV>(X, rows, cols, ldx, comps, ldcomp, plane, ws, slot, blockIdx.x, blockIdx.y, gridDim.y, red);
 }
 
@@ -101,11 +101,11 @@ template <int NLEV>
 __device__ __forceinline__ void f64_spec_transpose_body(const double *__restrict__ X, int64_t rows, int64_t cols,
                                                         int64_t ldx, uint16_t *__restrict__ comps, int64_t ldcomp,
                                                         int64_t plane, WsHeader *ws, int slot, int64_t bid,
-                                                        int64_t nblk, uint32_t *smw, unsigned long long *red)
+                                                        int64_t nblk, uint32_t *smw, uint32_t *red)
 {
     const int v0 = spec_v0(ws, slot);
     const bool fast = v0 >= -78;
-    float P[6] = {};
+    float P[3] = {};
     if (fast) spec_units(v0 - 50, P);
     const bool vin = ((ldx & 1) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
     const bool vout = ((ldcomp & 7) == 0) && ((plane & 7) == 0) && ((reinterpret_cast<uintptr_t>(comps) & 15u) == 0);
@@ -187,7 +187,7 @@ f64_spec_transpose_kernel(const double *__restrict__ X, int64_t rows, int64_t co
                           uint16_t *__restrict__ comps, int64_t ldcomp, int64_t plane, WsHeader *ws, int slot)
 {
     extern __shared__ __align__(16) uint32_t smw[];                  // [6][kTile][kTile / 2]
-    __shared__ unsigned long long red[5 * (kThreads / 32)];
+    __shared__ uint32_t red[5 * (kThreads / 32)];
     f64_spec_transpose_body<NLEV>(X, rows, cols, ldx, comps, ldcomp, plane, ws, slot, blockIdx.x, gridDim.x, smw, red);
 }
 

@@ -115,25 +115,18 @@ __global__ void rc_levels_kernel(int L, unsigned long long *maxbits, int32_t *vr
 // Speculative pass with per-vector levels: each element is split with its
 // vector's v0 (level 0 is literal) under the assumption v^(r) = v0 - 8r, as
 // in the whole-matrix speculative pass; the magnitudes |X^(r)| before levels
-// 1 .. 5 are reduced per vector into vmax[5][vectors] (32-bit: levels 1 and
-// 2 in units of 2^(F + 20) with a sticky last bit, levels 3 .. 5 exact in
-// units of 2^F, F = v0 - 50).
-__device__ __forceinline__ uint32_t jam20(unsigned long long m)
-{
-    return (uint32_t)(m >> 20) | ((m & 0xFFFFFull) != 0 ? 1u : 0u);
-}
-
-__device__ __forceinline__ void spec_element_mags(double x, int v0, const float (&P)[6], uint32_t (&s)[6],
-                                                  uint32_t &badmask, uint32_t (&mag)[5])
+// 1 .. 5 are reduced per vector into vmax[5][vectors] (bits of non-negative
+// FP32 values in the units of kMagShift).
+__device__ __forceinline__ void spec_element_mags(double x, int v0, const float (&P)[3], uint32_t (&s)[6],
+                                                  uint32_t &badmask, float (&mag)[5])
 {
     SpecState st;
+#pragma unroll
+    for (int r = 0; r < 5; ++r) st.m[r] = mag[r];
     spec_element(x, v0, v0 >= -78, P, s, st);
     badmask |= st.badmask;
-    mag[0] = jam20(st.m1);
-    mag[1] = jam20(st.m2);
-    mag[2] = st.m[0];
-    mag[3] = st.m[1];
-    mag[4] = st.m[2];
+#pragma unroll
+    for (int r = 0; r < 5; ++r) mag[r] = st.m[r];
 }
 
 // Row-major planes, levels per row: thread = 4 consecutive entries of a row.
@@ -149,7 +142,7 @@ rc_spec_rows_kernel(const double *__restrict__ X, int64_t rows, int64_t cols, in
     uint32_t badmask = 0;
     for (int64_t i = blockIdx.y; i < rows; i += gridDim.y) {
         const int v0 = vrc[i];
-        uint32_t mx[5] = {0, 0, 0, 0, 0};
+        float mx[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         if (j0 < cols) {
             const double *src = X + i * ldx + j0;
             double x[4];
@@ -160,19 +153,14 @@ rc_spec_rows_kernel(const double *__restrict__ X, int64_t rows, int64_t cols, in
 #pragma unroll
                 for (int e = 0; e < 4; ++e) x[e] = (j0 + e < cols) ? src[e] : 0.0;
             }
-            float P[6] = {};
+            float P[3] = {};
             if (v0 >= -78) spec_units(v0 - 50, P);
             uint32_t w[6][2];
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
-                uint32_t sa[6], sb[6], ma[5], mb[5];
-                spec_element_mags(x[e], v0, P, sa, badmask, ma);
-                spec_element_mags(x[e + 1], v0, P, sb, badmask, mb);
-#pragma unroll
-                for (int r = 0; r < 5; ++r) {
-                    const uint32_t mm = ma[r] > mb[r] ? ma[r] : mb[r];
-                    mx[r] = mm > mx[r] ? mm : mx[r];
-                }
+                uint32_t sa[6], sb[6];
+                spec_element_mags(x[e], v0, P, sa, badmask, mx);
+                spec_element_mags(x[e + 1], v0, P, sb, badmask, mx);
 #pragma unroll
                 for (int r = 0; r < 6; ++r) w[r][e >> 1] = pack2(sa[r], sb[r]);
             }
@@ -190,7 +178,7 @@ rc_spec_rows_kernel(const double *__restrict__ X, int64_t rows, int64_t cols, in
         }
 #pragma unroll
         for (int r = 0; r < 5; ++r) {
-            const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, mx[r]);
+            const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx[r]));
             if (lane_id() == 0 && m) atomicMax(&vmax[r * rows + i], m);
         }
     }
@@ -235,16 +223,17 @@ rc_spec_transpose_kernel(const double *__restrict__ X, int64_t rows, int64_t col
             for (int e = 0; e < 2; ++e) {
                 const int64_t col = gj + k + e;
                 const int v0 = col < cols ? vrc[col] : kZeroLevel;
-                float P[6] = {};
+                float P[3] = {};
                 if (v0 >= -78) spec_units(v0 - 50, P);
-                uint32_t s0[6], s1[6], m0[5], m1[5];
-                spec_element_mags(x[0][e], v0, P, s0, badmask, m0);
-                spec_element_mags(x[1][e], v0, P, s1, badmask, m1);
+                uint32_t s0[6], s1[6];
+                float mx[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+                spec_element_mags(x[0][e], v0, P, s0, badmask, mx);
+                spec_element_mags(x[1][e], v0, P, s1, badmask, mx);
 #pragma unroll
                 for (int r = 0; r < 6; ++r) smw[(r * kTile + 8 * q + k + e) * (kTile / 2) + p] = pack2(s0[r], s1[r]);
 #pragma unroll
                 for (int r = 0; r < 5; ++r) {
-                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, m0[r] > m1[r] ? m0[r] : m1[r]);
+                    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx[r]));
                     if (p == 0 && m && col < cols) atomicMax(&vmax[r * cols + col], m);
                 }
             }
@@ -274,7 +263,8 @@ rc_spec_transpose_kernel(const double *__restrict__ X, int64_t rows, int64_t col
     if (badmask && lane_id() == 0) atomicOr(&ws->slice_bad[slot], badmask);
 }
 
-__device__ __forceinline__ int ceil_log2_u32(uint32_t m) { return m <= 1u ? 0 : 32 - __clz(m - 1u); }
+// ceil(log2) of a positive FP32 value of at least 1/2, given by its bits.
+__device__ __forceinline__ int ceil_log2_f32(uint32_t b) { return (int)(b >> 23) - 127 + ((b & 0x7FFFFFu) ? 1 : 0); }
 
 // One thread per vector: checks its speculative levels in order.  A level
 // that matches v0 - 8r is final (the 32-bit maxima decide matches exactly);
@@ -302,7 +292,7 @@ __device__ __forceinline__ void rc_verify_pass(const uint32_t *vmax, int32_t *vr
                 if (zero) { vrc[r * nvec + i] = kZeroLevel; continue; }
                 const uint32_t m = vmax[(r - 1) * nvec + i];
                 if (m == 0) { vrc[r * nvec + i] = kZeroLevel; zero = true; continue; }
-                const int vr = ceil_log2_u32(m) + F + (r <= 2 ? 20 : 0);
+                const int vr = ceil_log2_f32(m) + F + kMagShift[r - 1];
                 if (vr != v0 - 8 * r) { f = r - 1; break; }
                 vrc[r * nvec + i] = vr;
             }
