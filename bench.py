@@ -235,7 +235,7 @@ class Case:
         # kernels of ours per step: FP32 split of both operands = 1 launch; FP64 split of both =
         # 5 (level maxima of both, then a speculative pass and a verifier per operand);
         # product-sum = 1, or 2 when the library runs the last partial wave of its widest
-        # tiles as 128 x 128 tiles (it reports its schedule)
+        # tiles as narrower ones (it reports its schedule)
         self.launches = 1 if self.fused else 1 + emu.emu_prodsum_f32_launches(M, N) if self.mode == 32 else \
             5 + emu.emu_prodsum_f64_launches(M, N)
         if self.merge_from is not None:

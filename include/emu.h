@@ -320,11 +320,11 @@ int emu_prodsum_f32_tile_rows(int64_t M, int64_t N);
 int emu_prodsum_f32_launches(int64_t M, int64_t N);
 
 /* Output-tile shape that the FP64-mode product-sum picks for an M x N
- * result, unless EMU_F64_TILE (128x64, 128x128, 128x256 or 256x256) forces one:
- * width 64, 128 or 256 columns; height 128 rows, or 256 rows where a 256-column
- * tile runs on a pair of SMs (a cluster of two CTAs sharing each MMA); and
- * the number of kernel launches (2 when the last, partial wave of 256-row
- * tiles runs as 128 x 128 tiles in a second launch).  The paper has no
+ * result, unless EMU_F64_TILE (128x64, 128x128, 256x128, 128x256 or 256x256)
+ * forces one: width 64, 128 or 256 columns; height 128 rows, or 256 rows where
+ * a tile runs on a pair of SMs (a cluster of two CTAs sharing each MMA); and the
+ * number of kernel launches (2 when the last, partial wave of 256 x 256 tiles
+ * runs as 256 x 128 ones in a second launch).  The paper has no
  * counterpart: every shape gives identical results, and the calls only
  * report which kernels run.  0 for sizes < 1. */
 int emu_prodsum_f64_tile_columns(int64_t M, int64_t N);

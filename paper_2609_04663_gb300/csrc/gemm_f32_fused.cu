@@ -90,7 +90,7 @@ gemm_f32_fused_kernel(const float *__restrict__ A, int64_t lda, const float *__r
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane_id() == 0) mma_loop<BN, KB, STAGES>(tmem, base, full0, empty0, accum_bar, nkb, flags);
+        mma_loop<BN, KB, STAGES>(tmem, base, full0, empty0, accum_bar, nkb, flags);
     } else {
         const int ct = threadIdx.x - 32;
         const int a_c4 = ct & 7, a_r0 = ct >> 3;

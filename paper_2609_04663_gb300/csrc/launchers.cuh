@@ -96,9 +96,9 @@ cudaError_t launch_prodsum_tail(int64_t M, int64_t N, int64_t K, const uint16_t 
                                 cudaStream_t st);
 
 // How the FP64 product-sum covers an M x N result: tiles of rows x cols
-// (128 x 64, 128 x 128, 128 x 256, or 256 x 256 on CTA pairs), `tiles` of them
-// in the first launch and, when launches == 2, the remaining ones as `rest`
-// 128 x 128 quarters in a second launch.
+// (128 x 64, 128 x 128, 128 x 256, or on CTA pairs 256 x 128 or 256 x 256),
+// `tiles` of them in the first launch and, when launches == 2, the remaining
+// ones as `rest` 256 x 128 halves in a second launch.
 struct F64Plan {
     int rows = 0, cols = 0, launches = 0;
     int64_t tiles = 0, rest = 0;
@@ -108,9 +108,9 @@ F64Plan f64_plan(int64_t M, int64_t N);
 int f64_tile_columns(int64_t M, int64_t N);
 // The FP64 product-sum kernel (prodsum_f64w_kernel.cuh): the first `tiles` tiles
 // in raster order of 128 x 256, or with pair of 256 x 256 on clusters of two
-// CTAs (launch_prodsum_f64_wide); of 128 x cols, cols = 128 or 64, or with
-// wide_first >= 0 `tiles` 128 x 128 quarters of the 256 x 256 tiles from raster
-// index wide_first on (launch_prodsum_f64_narrow).  acc: f64_acc_bytes(M, N)
+// CTAs (launch_prodsum_f64_wide); of 128 x cols, cols = 128 or 64, or with pair
+// of 256 x 128, with wide_first >= 0 `tiles` halves of the 256 x 256 tiles from
+// raster index wide_first on (launch_prodsum_f64_narrow).  acc: f64_acc_bytes(M, N)
 // bytes.
 cudaError_t launch_prodsum_f64_wide(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp,
                                      int64_t ldcomp, const int32_t *vA, const int32_t *vB, int nprod, double *C,
@@ -119,7 +119,7 @@ cudaError_t launch_prodsum_f64_wide(int64_t M, int64_t N, int64_t K, const uint1
 cudaError_t launch_prodsum_f64_narrow(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp,
                                      int64_t ldcomp, const int32_t *vA, const int32_t *vB, int nprod, double *C,
                                      int64_t ldc, double *acc, uint32_t *flags, cudaStream_t st, int64_t a_plane,
-                                     bool rowcol, const float *T, int64_t ldt, int cols, int64_t tiles,
+                                     bool rowcol, const float *T, int64_t ldt, int cols, bool pair, int64_t tiles,
                                       int wide_first);
 
 // Bytes of the FP64 product-sum's accumulator, enough for either tile shape:

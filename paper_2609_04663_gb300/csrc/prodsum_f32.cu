@@ -175,7 +175,7 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             ++issued;
         }
         if (!ok) drain_inflight(full0, STAGES, issued, flags);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         mma_loop<BN, KB, STAGES>(tmem, base, full0, empty0, accum_bar, nkb, flags);
     } else if (warp >= 2) {
         // ---------------- epilogue: TMEM -> registers -> C (tcgen05.ld needs the
@@ -293,28 +293,20 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 while (globaltimer_ns() - t0 < 200000ull) {}
             }
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 1 && rank == 0) {
         // ---------------- MMA issuer (the leader): the six products of Eq.
-        // (fp32reuseorder) per 16-wide K step, M = 256 over the pair
+        // (fp32reuseorder) per 16-wide K step, M = 256 over the pair (the warp walks
+        // the loop together and one elected lane issues, as in mma_loop)
         constexpr uint32_t idesc = make_idesc_bf16(2 * kBM, BN);
         for (int kb = 0; kb < nkb; ++kb) {
             const int s = kb % STAGES;
-            if (!mbar_wait(full0 + 8u * s, (kb / STAGES) & 1, flags)) break;
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * s, (kb / STAGES) & 1, flags))) break;
             tc_fence_after();
-            const uint32_t st = base + (uint32_t)(s * Cfg::STAGE);
-#pragma unroll
-            for (int kk = 0; kk < KB / 16; ++kk) {
-#pragma unroll
-                for (int q = 0; q < 6; ++q) {
-                    const uint64_t ad = make_sdesc(st + kChain[q][0] * Cfg::A_TILE + kk * 32, Cfg::SBO, Cfg::SWZ);
-                    const uint64_t bd = make_sdesc(st + 3 * Cfg::A_TILE + kChain[q][1] * Cfg::B_TILE + kk * 32,
-                                                   Cfg::SBO, Cfg::SWZ);
-                    mma_bf16_pair(tmem, ad, bd, idesc, (kb | kk | q) != 0);
-                }
-            }
-            mma_commit_pair(empty0 + 8u * s);         // both CTAs' stages reusable once these finish
+            issue_products<Cfg, KB, Cfg::B_TILE, true>(tmem, base + (uint32_t)(s * Cfg::STAGE), idesc, kb != 0,
+                                                       empty0 + 8u * s);       // both CTAs' stages reusable then
         }
-        mma_commit_pair(accum_bar);                   // both CTAs' accumulator parts complete
+        if (elect_one()) mma_commit_pair(accum_bar);  // both CTAs' accumulator parts complete
+        __syncwarp();
     } else if (warp >= 2) {
         // ---------------- epilogue of this CTA's 128 rows (tcgen05.ld needs the
         // whole warp, so a timeout in any lane skips the warp's epilogue)

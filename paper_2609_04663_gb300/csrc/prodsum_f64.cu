@@ -11,21 +11,25 @@ constexpr int kTileRows = 128;
 
 // Tile shape of the FP64 product-sum.  Every shape forms the same exact sums
 // and adds them with the same roundings, so C does not depend on the choice.
-// Measured per-SM rates relative to 256 x 256 tiles on CTA pairs (4096^3, 21
-// products, every SM busy): 128 x 256 0.95, 128 x 128 0.75, 128 x 64 0.41; a
-// narrower tile brings more operand bytes into the SM per FLOP.
-// - The shape with the least waves x columns / rate is taken; 256 x 256 needs
-//   two 128-row tile rows and replaces 128 x 256 then.
-// - 64-column tiles are taken where 128 x 128 ones would leave more than 60 % of
-//   the SMs idle: with so few CTAs the time is that of one CTA's chain of
+// Per-SM rates relative to 256 x 256 tiles on CTA pairs (4096^3, 21 products,
+// every SM busy, 1446 TFLOP/s): 256 x 128 on pairs 0.82, 128 x 256 0.85, 128 x 128
+// 0.68, 128 x 64 0.39; a narrower tile moves more operand bytes through shared
+// memory per FLOP.  (A single wave of 256 x 128 tiles takes a little more than
+// the rate says: kRateHalf.)
+// - The shape with the least waves x columns / rate is taken.  Pairs need two
+//   128-row tile rows.
+// - 128 x 128 tiles are taken only where 256 x 128 pairs would leave half of the
+//   SMs idle or more, and 64-column tiles where 128 x 128 ones would leave more
+//   than 60 % idle: with so few CTAs the time is that of one CTA's chain of
 //   products, which is shorter for half the columns (256^3, 21 products: 40
-//   against 54 us; 3001 x 203 x 2999: 300 against 380 us).
+//   against 54 us; 3001 x 203 x 2999: 283 against 378 us).
 // - When 256 x 256 tiles leave the last wave partly empty, the full waves run
-//   as such and a second launch takes the remaining tiles as 128 x 128 quarters,
-//   if that is estimated faster.
-// EMU_F64_TILE=128x64 / 128x128 / 128x256 / 256x256 forces one shape for every
-// result (and no mixed last wave).
-constexpr double kRateQuarter = 0.75;
+//   as such and a second launch takes the remaining tiles as 256 x 128 halves,
+//   if that is estimated faster (4096^3, 21 products: 1996 us in four waves,
+//   1901 us as three and one of halves).
+// EMU_F64_TILE=128x64 / 128x128 / 256x128 / 128x256 / 256x256 forces one shape
+// for every result (and no mixed last wave).
+constexpr double kRateHalf = 0.75;
 static int f64_tile_forced()
 {
     static const int forced = [] {
@@ -33,8 +37,9 @@ static int f64_tile_forced()
         if (!e) return 0;
         if (std::strcmp(e, "256x256") == 0) return 1;
         if (std::strcmp(e, "128x256") == 0) return 2;
-        if (std::strcmp(e, "128x128") == 0) return 3;
-        if (std::strcmp(e, "128x64") == 0) return 4;
+        if (std::strcmp(e, "256x128") == 0) return 3;
+        if (std::strcmp(e, "128x128") == 0) return 4;
+        if (std::strcmp(e, "128x64") == 0) return 5;
         return 0;
     }();
     return forced;
@@ -57,13 +62,17 @@ F64Plan f64_plan(int64_t M, int64_t N)
     const int sms = device_sms();
     const int64_t tiles_m = (M + kTileRows - 1) / kTileRows;
     struct Shape { int rows, cols; double rate; };
-    static const Shape shapes[4] = {{256, 256, 1.0}, {128, 256, 0.95}, {128, 128, kRateQuarter}, {128, 64, 0.41}};
+    static const Shape shapes[5] = {
+        {256, 256, 1.0}, {128, 256, 0.85}, {256, 128, kRateHalf}, {128, 128, 0.66}, {128, 64, 0.38}};
     const bool few = tiles_m * ((N + 127) / 128) * 10 < (int64_t)sms * 4;
+    // 128-column tiles of 128 rows only where pairs would leave half of the SMs idle
+    const bool few_pairs = ((tiles_m + 1) / 2) * ((N + 127) / 128) * 4 <= (int64_t)sms || tiles_m < 2;
     p.launches = 1;
     double best = 0.0;
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 5; ++i) {
         const Shape &h = shapes[i];
-        if (forced ? forced != i + 1 : (h.cols == 256 && (h.rows == 256) != (tiles_m >= 2)) || (h.cols == 64 && !few))
+        if (forced ? forced != i + 1 : (h.cols == 256 && (h.rows == 256) != (tiles_m >= 2)) ||
+                         (h.rows == 256 && tiles_m < 2) || (h.cols == 128 && (h.rows == 256) == few_pairs) || (h.cols == 64 && !few))
             continue;
         const int64_t tiles = ((M + h.rows - 1) / h.rows) * ((N + h.cols - 1) / h.cols);
         const int64_t slots = sms / (h.rows / kTileRows);
@@ -78,10 +87,10 @@ F64Plan f64_plan(int64_t M, int64_t N)
     if (!forced && p.rows == 256) {
         const int64_t slots = sms / 2, full = (p.tiles / slots) * slots, rem = p.tiles - full;
         const double t_mixed =
-            (double)(full / slots) * 256.0 + (double)((4 * rem + sms - 1) / sms) * 128.0 / kRateQuarter;
+            (double)(full / slots) * 256.0 + (double)((2 * rem + slots - 1) / slots) * 128.0 / kRateHalf;
         if (full > 0 && rem > 0 && t_mixed < 0.97 * best) {
             p.tiles = full;
-            p.rest = 4 * rem;
+            p.rest = 2 * rem;
             p.launches = 2;
         }
     }
@@ -101,12 +110,12 @@ cudaError_t launch_prodsum_f64(int64_t M, int64_t N, int64_t K, const uint16_t *
     const F64Plan p = f64_plan(M, N);
     if (p.cols < 256)
         return launch_prodsum_f64_narrow(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
-                                         rowcol, T, ldt, p.cols, p.tiles, -1);
+                                         rowcol, T, ldt, p.cols, p.rows == 256, p.tiles, -1);
     cudaError_t e = launch_prodsum_f64_wide(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
                                             rowcol, T, ldt, p.rows == 256, p.tiles);
     if (e != cudaSuccess || p.rest == 0) return e;
     return launch_prodsum_f64_narrow(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane, rowcol, T,
-                                     ldt, 128, p.rest, (int)p.tiles);
+                                     ldt, 128, true, p.rest, (int)p.tiles);
 }
 
 }  // namespace emu

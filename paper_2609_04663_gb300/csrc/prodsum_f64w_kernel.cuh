@@ -8,10 +8,10 @@
 // integer of at most 2^24 units u = 2^(vA_i + vB_j - 16).
 //
 // Output tiles are 128 rows by BN = 256, 128 or 64 columns per CTA, or (PAIR)
-// 256 x 256 on a cluster of two CTAs of one TPC with cta_group::2 MMAs (M =
-// 256): each CTA stages its 128 rows of the A slice and half of the B slice's
-// 256 rows, the leader (cluster rank 0) issues the MMAs for both, and each
-// CTA's TMEM receives its 128 x 256 part of the partials.  Every MMA brings
+// 256 x 256 or 256 x 128 on a cluster of two CTAs of one TPC with cta_group::2
+// MMAs (M = 256): each CTA stages its 128 rows of the A slice and half of the B
+// slice's BN rows, the leader (cluster rank 0) issues the MMAs for both, and each
+// CTA's TMEM receives its 128 x BN part of the partials.  Every MMA brings
 // its operands into the SM through shared memory and for one product at a
 // time nothing is reused across MMAs, so wider tiles move fewer bytes per
 // FLOP (per 2^20 FLOP: 8 KB as a pair, 12 KB at 256 columns, 16 KB at 128,
@@ -136,6 +136,14 @@ __device__ __forceinline__ void drain_barrier()
     asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory");
 }
 
+// max(|a|, |b|, |c|)
+__device__ __forceinline__ float max3_abs(float a, float b, float c)
+{
+    float r;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // FP64 reduction in L2: *p <- fl64(*p + x), round to nearest even.
 __device__ __forceinline__ void red_add_f64(double *p, double x)
 {
@@ -154,6 +162,9 @@ struct LevelSummary {
     int lock;                    // every vector's levels fall in steps of 8
     int min_a, max_a, min_b, max_b;
 };
+
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld32(taddr, r); }
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld16(taddr, r); }
 
 // Levels v[0 .. d-1] (stride apart) of one matrix or vector: how far the
 // finest level lies below v_0 - 8r (0: steps of 8 until the residual is zero).
@@ -197,8 +208,8 @@ __device__ __forceinline__ float start_of(uint32_t code, uint32_t bound_bits)
 }
 
 // TAIL: add the merged tail T (an M x N FP32 matrix) once after the last product.
-// wide_first >= 0 (BN = 128): this launch takes the 128 x 128 quarters of the
-// 256 x 256 tiles from raster index wide_first on.
+// wide_first >= 0 (pairs with BN = 128): this launch takes the 256 x 128 halves
+// of the 256 x 256 tiles from raster index wide_first on.
 template <int BN, bool ROWCOL, bool TAIL, bool PAIR>
 __global__ void __launch_bounds__(F64WCfgT<BN, PAIR>::THREADS, 1)
 prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -224,16 +235,17 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     int tm, tn;
     if constexpr (PAIR) {                             // the pair's 256 rows: this CTA takes half `rank`
         int tp;
-        tile_coords((int)(blockIdx.x >> 1), (M + 2 * kBM - 1) / (2 * kBM), tiles_n, tp, tn);
+        const int pair = (int)(blockIdx.x >> 1), tiles_p = (M + 2 * kBM - 1) / (2 * kBM);
+        if (BN == 128 && wide_first >= 0) {
+            // the two column halves of each 256 x 256 tile that a last, partial wave would have taken
+            int tnw;
+            tile_coords(wide_first + (pair >> 1), tiles_p, (N + 255) / 256, tp, tnw);
+            tn = 2 * tnw + (pair & 1);
+            if (tn >= tiles_n) return;                // past the last column (both CTAs)
+        } else {
+            tile_coords(pair, tiles_p, tiles_n, tp, tn);
+        }
         tm = 2 * tp + (int)rank;
-    } else if (BN == 128 && wide_first >= 0) {
-        // the four 128 x 128 quarters of each 256 x 256 tile that a last, partial wave would have taken
-        const int tiles_m = (M + kBM - 1) / kBM, quarter = (int)(blockIdx.x & 3);
-        int tp, tnw;
-        tile_coords(wide_first + (int)(blockIdx.x >> 2), (tiles_m + 1) / 2, (N + 255) / 256, tp, tnw);
-        tm = 2 * tp + (quarter >> 1);
-        tn = 2 * tnw + (quarter & 1);
-        if (tm >= tiles_m || tn >= tiles_n) return;   // a quarter past the last row or column
     } else {
         tile_coords(blockIdx.x, (M + kBM - 1) / kBM, tiles_n, tm, tn);
     }
@@ -306,8 +318,11 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 while (globaltimer_ns() - t0 < 200000ull) {}
             }
         }
-      } else if (warp == 1 && lane == 0 && rank == 0) {
-        // ---------------- MMA issuer (a pair's leader): one chunk partial into buffer t % NBUF
+      } else if (warp == 1 && rank == 0) {
+        // ---------------- MMA issuer (a pair's leader): one chunk partial into buffer t % NBUF.
+        // The whole warp walks the loop (waits decided by vote), one elected lane
+        // issues: control flow and operands are then uniform, and the descriptors
+        // need no move from vector to uniform registers before every MMA.
         constexpr uint32_t idesc = make_idesc_bf16(PAIR ? 2 * kBM : kBM, BN);
         // descriptors of stage 0; stage s and 16-wide K step kk add (s STAGE + 32 kk) / 16
         const uint64_t ad0 = make_sdesc(base, Cfg::SBO, Cfg::SWZ), bd0 = make_sdesc(base + Cfg::A_TILE, Cfg::SBO, Cfg::SWZ);
@@ -316,32 +331,38 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         bool ok = true;
         for (int t = 0; t < nprod * nch && ok; ++t) {
             const int kbs = min(kKChunk / Cfg::KB, (K - c * kKChunk + Cfg::KB - 1) / Cfg::KB);
-            if (!(ok = mbar_wait(tempty0 + 8u * b, tph ^ 1u, flags))) break;
+            if (!(ok = __all_sync(0xFFFFFFFFu, mbar_wait(tempty0 + 8u * b, tph ^ 1u, flags)))) break;
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(b * BN);
             for (int u = 0; u < kbs; ++u) {
-                if (!(ok = mbar_wait(full0 + 8u * s, ph, flags))) break;
+                if (!(ok = __all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * s, ph, flags)))) break;
                 tc_fence_after();
                 const uint32_t off = (uint32_t)(s * (Cfg::STAGE / 16));
+                const uint64_t ad = ad0 + off, bd = bd0 + off;
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < Cfg::KB / 16; ++kk) {
-                    const uint64_t ad = ad0 + (off + 2 * kk), bd = bd0 + (off + 2 * kk);
-                    if constexpr (PAIR) mma_bf16_pair(d, ad, bd, idesc, (u | kk) != 0);
-                    else mma_bf16(d, ad, bd, idesc, (u | kk) != 0);
+                    for (int kk = 0; kk < Cfg::KB / 16; ++kk) {
+                        if constexpr (PAIR) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (u | kk) != 0);
+                        else mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (u | kk) != 0);
+                    }
+                    if constexpr (PAIR) mma_commit_pair(empty0 + 8u * s);
+                    else mma_commit(empty0 + 8u * s);
+                    if (u + 1 == kbs) {
+                        if constexpr (PAIR) mma_commit_pair(tfull0 + 8u * b);
+                        else mma_commit(tfull0 + 8u * b);
+                    }
                 }
-                if constexpr (PAIR) mma_commit_pair(empty0 + 8u * s);
-                else mma_commit(empty0 + 8u * s);
+                __syncwarp();
                 if (++s == Cfg::STAGES) { s = 0; ph ^= 1u; }
-            }
-            if (ok) {
-                if constexpr (PAIR) mma_commit_pair(tfull0 + 8u * b);
-                else mma_commit(tfull0 + 8u * b);
             }
             if (++b == Cfg::NBUF) { b = 0; tph ^= 1u; }
             if (++c == nch) c = 0;
         }
-        if constexpr (PAIR) mma_commit_pair(done_bar);
-        else mma_commit(done_bar);
+        if (elect_one()) {
+            if constexpr (PAIR) mma_commit_pair(done_bar);
+            else mma_commit(done_bar);
+        }
+        __syncwarp();
         (void)mbar_wait(done_bar, 0, flags);
       }
     } else {
@@ -490,42 +511,66 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 __syncwarp();
                 if (!ok) break;
                 tc_fence_after();
-                constexpr int LD = Cfg::COLS >= 32 && !(ROWCOL && BN == 256) ? 32 : 16;      // columns per TMEM load
-                uint32_t pv[LD];                                  // the partials
+                // LD columns at a time, the next LD on their way from TMEM meanwhile.  The sums
+                // replace the partials in their registers; the largest magnitudes are found in
+                // independent chains and voted on once (one chain of compares, each waiting
+                // for the last, and a vote per 16 columns took as long as the MMAs).
+                constexpr int LD = Cfg::COLS >= 32 ? 32 : 16;
+                uint32_t pv[2][LD];
+                tmem_ld_cols(tcol + (uint32_t)(b * BN), pv[0]);
 #pragma unroll
-                for (int h = 0; h < Cfg::COLS; h += 16) {
-                    const uint32_t taddr = tcol + (uint32_t)(b * BN + h);
-                    if (h % LD == 0) {
-                        if constexpr (LD == 32) tmem_ld32(taddr, pv);
-                        else tmem_ld16(taddr, pv);
-                        tmem_ld_wait();
-                    }
-                    float v[16];                                  // the sums
-                    bool big = false;
-                    if constexpr (ROWCOL) {
+                for (int hl = 0; hl < Cfg::COLS; hl += LD) {
+                    uint32_t (&ps)[LD] = pv[(hl / LD) & 1];
+                    tmem_ld_wait();
+                    if (hl + LD < Cfg::COLS) tmem_ld_cols(tcol + (uint32_t)(b * BN + hl + LD), pv[(hl / LD + 1) & 1]);
+                    bool big[LD / 16];
 #pragma unroll
-                        for (int j = 0; j < 16; j += 4) {
-                            const int4 f = *reinterpret_cast<const int4 *>(lvl + h + j);
-                            const int lv[4] = {f.x, f.y, f.z, f.w};
+                    for (int g = 0; g < LD; g += 16) {
+                        if constexpr (ROWCOL) {
+                            int mx[4] = {-0x7FFFFFFF, -0x7FFFFFFF, -0x7FFFFFFF, -0x7FFFFFFF};
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                v[j + k] = __fadd_rn(hi[h + j + k], __uint_as_float(pv[h % LD + j + k]));
-                                big |= (int)(__float_as_uint(v[j + k]) & 0x7FFFFFFFu) >= lv[k] + abits_lim;
+                            for (int j = g; j < g + 16; j += 4) {
+                                const int4 f = *reinterpret_cast<const int4 *>(lvl + hl + j);
+                                const int lv[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) {
+                                    ps[j + k] = __float_as_uint(__fadd_rn(hi[hl + j + k], __uint_as_float(ps[j + k])));
+                                    mx[k] = max(mx[k], (int)(ps[j + k] & 0x7FFFFFFFu) - lv[k]);
+                                }
                             }
-                        }
-                    } else {
+                            big[g / 16] = max(max(mx[0], mx[1]), max(mx[2], mx[3])) >= abits_lim;
+                        } else {
+                            float mx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            v[j] = __fadd_rn(hi[h + j], __uint_as_float(pv[h % LD + j]));
-                            big |= !(fabsf(v[j]) < limit);
+                            for (int j = g; j < g + 16; j += 2) {
+                                const float s0 = __fadd_rn(hi[hl + j], __uint_as_float(ps[j]));
+                                const float s1 = __fadd_rn(hi[hl + j + 1], __uint_as_float(ps[j + 1]));
+                                mx[(j >> 1) & 3] = max3_abs(mx[(j >> 1) & 3], s0, s1);
+                                ps[j] = __float_as_uint(s0);
+                                ps[j + 1] = __float_as_uint(s1);
+                            }
+                            big[g / 16] = !(max3_abs(max3_abs(mx[0], mx[1], mx[2]), mx[3], 0.0f) < limit);
                         }
                     }
-                    if (!__any_sync(0xFFFFFFFFu, big)) {
+                    if (!__any_sync(0xFFFFFFFFu, big[0] || big[LD / 16 - 1])) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) hi[h + j] = v[j];
-                    } else if (carry) {
+                        for (int j = 0; j < LD; ++j) hi[hl + j] = __uint_as_float(ps[j]);
+                        continue;
+                    }
+#pragma unroll
+                    for (int g = 0; g < LD; g += 16) {
+                    const int h = hl + g;
+                    uint32_t p16[16];                             // the partials again
+                    if (!__any_sync(0xFFFFFFFFu, big[g / 16])) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) hi[h + j] = __uint_as_float(ps[g + j]);
+                        continue;
+                    }
+                    tmem_ld16(tcol + (uint32_t)(b * BN + h), p16);
+                    tmem_ld_wait();
+                    if (carry) {
                         // rare: some sum would reach 2^24 u.  Split the running sum and
-                        // the partial at multiples of 2^12 u by the add-subtract
+                        // the partial (read again from TMEM) at multiples of 2^12 u by the add-subtract
                         // projection; the coarse parts go to the low word in C, the
                         // remainders (below 2^12 u) restart the running sum.  All exact.
                         const bool was = (dirty >> (h / 16)) & 1u;
@@ -536,7 +581,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                         for (int jj = 0; jj < 16; ++jj) {
                             const int j = h + jj;
-                            const float p = __uint_as_float(pv[h % LD + jj]);
+                            const float p = __uint_as_float(p16[jj]);
                             const float h1 = __fsub_rn(__fadd_rn(hi[j], cm), cm), l1 = __fsub_rn(hi[j], h1);
                             const float h2 = __fsub_rn(__fadd_rn(p, cm), cm), l2 = __fsub_rn(p, h2);
                             hi[j] = __fadd_rn(l1, l2);
@@ -555,7 +600,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                         for (int jj = 0; jj < 16; ++jj) {
                             const int j = h + jj;
-                            const float p = __uint_as_float(pv[h % LD + jj]);
+                            const float p = __uint_as_float(p16[jj]);
                             float be = 0.0f;
                             if (ROWCOL && j < lim && nch <= 2048)
                                 be = bound_of_levels(a_row, vB[(int64_t)kDiag[q][1] * N + n0 + cq * Cfg::COLS + j]);
@@ -576,14 +621,13 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                             if (j < lim) lrow[2 * j] = lo[jj];
                         }
                     }
-                    if (h + 16 == Cfg::COLS) {                   // buffer free: all values are in registers
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) {
-                            if constexpr (PAIR) mbar_arrive_peer(peer_addr(tempty0 + 8u * b, 0));
-                            else mbar_arrive(tempty0 + 8u * b);
-                        }
                     }
+                }
+                tc_fence_before();                                // buffer free: all values are in registers
+                __syncwarp();
+                if (lane == 0) {
+                    if constexpr (PAIR) mbar_arrive_peer(peer_addr(tempty0 + 8u * b, 0));
+                    else mbar_arrive(tempty0 + 8u * b);
                 }
                 if (coded < Cfg::COLS && c >= 2) { code_columns(coded); coded += HC; }
             }
@@ -795,8 +839,8 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 
 // tiles: the first `tiles` tiles in raster order (all of them, or the full
 // waves when narrower tiles take the rest), one CTA each, or with PAIR one
-// cluster of two CTAs each; or with wide_first >= 0 (BN = 128) `tiles` 128 x 128
-// quarters of the 256 x 256 tiles from raster index wide_first on.
+// cluster of two CTAs each; or with wide_first >= 0 (pairs, BN = 128) `tiles`
+// 256 x 128 halves of the 256 x 256 tiles from raster index wide_first on.
 template <int BN, bool ROWCOL, bool TAIL, bool PAIR>
 cudaError_t run_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp, int64_t ldcomp,
                      const int32_t *vA, const int32_t *vB, int nprod, double *C, int64_t ldc, double *acc,
