@@ -233,11 +233,12 @@ class Case:
         self.flop = 2.0 * M * N * K
         self.exec_flop = self.flop * (6 if self.mode == 32 else self.nprod)
         # kernels of ours per step: FP32 split of both operands = 1 launch; FP64 split of both =
-        # 5 (level maxima of both, then a speculative pass and a verifier per operand);
+        # 4 (level maxima of both, a speculative pass per operand, the verifier of both), or 1
+        # for at most 2^22 entries;
         # product-sum = 1, or 2 when the library runs the last partial wave of its widest
         # tiles as narrower ones (it reports its schedule)
         self.launches = 1 if self.fused else 1 + emu.emu_prodsum_f32_launches(M, N) if self.mode == 32 else \
-            5 + emu.emu_prodsum_f64_launches(M, N)
+            (1 if (M + N) * K <= 1 << 22 else 4) + emu.emu_prodsum_f64_launches(M, N)
         if self.merge_from is not None:
             self.launches += 1                    # the tail kernel
         if self.api and self.mode == 32:

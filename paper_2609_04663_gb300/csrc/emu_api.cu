@@ -340,8 +340,8 @@ namespace {
 
 // Shared body of the general GEMMs: validation, the splits of op(A) and
 // op(B) into K-major planes (the split's transpose flag absorbs op), the
-// product-sum into C (alpha = 1, beta = 0) or into the workspace product
-// buffer followed by the epilogue.
+// product-sum into C (alpha = 1, beta = 0; FP32 mode: with alpha and beta in its
+// epilogue) or into the workspace product buffer followed by the epilogue.
 template <typename T>
 emu_status gemm_ex(int opA, int opB, int64_t M, int64_t N, int64_t K, T alpha, const T *A, int64_t lda, const T *B,
                    int64_t ldb, T beta, T *C, int64_t ldc, int nprod, void *ws, size_t ws_bytes, cudaStream_t st)
@@ -376,18 +376,19 @@ emu_status gemm_ex(int opA, int opB, int64_t M, int64_t N, int64_t K, T alpha, c
     } else {
         // op(A) -> planes [S][M][ldk]; op(B) -> planes [S][N][ldk]
         const bool ta = opA == EMU_OP_T, tb = opB == EMU_OP_N;
-        const int64_t ar = ta ? K : M, ac = ta ? M : K, br = tb ? K : N, bc = tb ? N : K;
         if constexpr (f64) {
             const int nlev = f64_diagonals(nprod);   // slices the product-sum uses
-            e = launch_split_f64(A, ar, ac, lda, ta, Ap, ldk, h->vout[0], h, 0, st, nlev);
-            if (e == cudaSuccess) e = launch_split_f64(B, br, bc, ldb, tb, Bp, ldk, h->vout[1], h, 1, st, nlev);
+            e = launch_split_f64_gemm(A, M, K, lda, B, N, ldb, Ap, Bp, ldk, h->vout[0], h->vout[1], h, st, nlev, ta, tb);
             if (e == cudaSuccess)
                 e = launch_prodsum_f64(M, N, K, Ap, Bp, ldk, h->vout[0], h->vout[1], nprod, out, ldo,
                                        gemm_acc(ws, M, N, K), &h->flags, st);
         } else {
-            e = launch_split_f32(A, ar, ac, lda, ta, Ap, ldk, h, st);
-            if (e == cudaSuccess) e = launch_split_f32(B, br, bc, ldb, tb, Bp, ldk, h, st);
-            if (e == cudaSuccess) e = launch_prodsum_f32(M, N, K, Ap, Bp, ldk, out, ldo, &h->flags, st);
+            // alpha and beta are applied by the product-sum's epilogue, straight into C
+            e = launch_split_f32_gemm(A, M, K, lda, B, N, ldb, Ap, Bp, ldk, h, nullptr, 0, st, ta, tb);
+            if (e == cudaSuccess)
+                e = launch_prodsum_f32(M, N, K, Ap, Bp, ldk, C, ldc, &h->flags, st, 0, 0, false, alpha, beta,
+                                       direct ? 0 : beta == T(0) ? 1 : 2);
+            return cuda_status(e);
         }
     }
     if (e == cudaSuccess && !direct) {

@@ -22,12 +22,14 @@ cudaError_t launch_split_f64(const double *X, int64_t rows, int64_t cols, int64_
                              uint16_t *comps, int64_t ldcomp, int32_t *v_out, WsHeader *ws, int slot,
                              cudaStream_t st, int nlev = 6);
 
-// Both operands of an FP64 GEMM split as launch_split_f64 splits A (rows x
-// cols = M x K, row-major planes, slot 0) and then B (K x N, K-major planes,
-// slot 1), with the level-maximum passes of the two sharing one launch.
+// Both operands of an FP64 GEMM split as launch_split_f64 splits op(A) (planes
+// of M rows, slot 0) and then op(B) (planes of N rows, slot 1), in fewer
+// launches (one for small operands); ta / tb: launch_split_f64's transpose of
+// the stored matrix.
 cudaError_t launch_split_f64_gemm(const double *A, int64_t M, int64_t K, int64_t lda, const double *B, int64_t N,
                                   int64_t ldb, uint16_t *Ap, uint16_t *Bp, int64_t ldcomp, int32_t *vA_out,
-                                  int32_t *vB_out, WsHeader *ws, cudaStream_t st, int nlev);
+                                  int32_t *vB_out, WsHeader *ws, cudaStream_t st, int nlev, bool ta = false,
+                                  bool tb = true);
 
 // Number of diagonals d of an FP64-mode product count (Eq. (fp64productcounts):
 // nprod = d (d + 1) / 2), i.e. the slices 0 .. d-1 a product-sum reads; 0 for
@@ -59,15 +61,19 @@ inline size_t rc_scratch_bytes(int64_t plane_rows) { return (size_t)plane_rows *
 // on its own.
 // c_zeroed: C is zero on entry, so when few output tiles would leave SMs idle
 // the product-sum may split K in two and add both halves into C.
+// ab: 0 = C <- P, 1 = C <- fl(alpha P), 2 = C <- fl(fl(alpha P) + fl(beta C)) (not
+// with c_zeroed).
 cudaError_t launch_prodsum_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp,
                                int64_t ldcomp, float *C, int64_t ldc, uint32_t *flags, cudaStream_t st,
-                               int64_t a_plane = 0, int64_t b_plane = 0, bool c_zeroed = false);
-// Both operands of an FP32 GEMM (A: M x K row-major planes, B: K x N K-major
-// planes, row pitch ldcomp, B's planes at Bp) split in one launch; with C
-// non-null the launch also sets the M x N result C (ldc) to zero.
+                               int64_t a_plane = 0, int64_t b_plane = 0, bool c_zeroed = false, float alpha = 1.0f,
+                               float beta = 0.0f, int ab = 0);
+// Both operands of an FP32 GEMM split in one launch: op(A) into planes of M rows,
+// op(B) into planes of N rows at Bp, row pitch ldcomp; ta / tb as for
+// launch_split_f64_gemm.  With C non-null the launch also sets the M x N result
+// C (ldc) to zero.
 cudaError_t launch_split_f32_gemm(const float *A, int64_t M, int64_t K, int64_t lda, const float *B, int64_t N,
                                   int64_t ldb, uint16_t *Ap, uint16_t *Bp, int64_t ldcomp, WsHeader *ws, float *C,
-                                  int64_t ldc, cudaStream_t st);
+                                  int64_t ldc, cudaStream_t st, bool ta = false, bool tb = true);
 // Tile width (256, 128 or 64) the FP32 product-sums pick for an M x N result,
 // and the number of K-parts (1 or 2) the product-sum takes when C is cleared
 // first.

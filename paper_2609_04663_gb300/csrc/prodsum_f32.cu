@@ -104,6 +104,48 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
     __syncwarp();
 }
 
+// Epilogue of one warp for a C that no tensor map describes, or with the
+// general GEMM's scaling (ab = 1: C <- fl(alpha P), ab = 2: C <- fl(fl(alpha P) +
+// fl(beta C)), each operation rounded once): each 32 x 32 piece is turned in
+// shared memory (stage memory, free once every MMA has completed; rows of 33
+// words, conflict-free both ways) so that a warp reads and writes whole row
+// segments, the rows of C it scales requested before the piece is read from
+// TMEM.  One lane per row, as in store_tile, touches a cache line per lane: at
+// 1537 x 2050 x 1100 that and a separate alpha / beta pass took 28 of 90 us.
+__device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int ncols, int m0, int n0, int M, int N,
+                                              float *__restrict__ C, int64_t ldc, float alpha, float beta, int ab,
+                                              uint8_t *stage)
+{
+    tc_fence_after();
+    const int lane = (int)lane_id(), row0 = m0 + quarter * 32, nr = min(32, M - row0);
+    float *buf = reinterpret_cast<float *>(stage) + quarter * (32 * 33);
+    const int cols = nr > 0 ? min(ncols, N - n0) : 0;
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 32) {
+        const bool mine = c + lane < cols;
+        float *cp = C + (int64_t)row0 * ldc + n0 + c + lane;
+        float old[32];
+        if (ab == 2) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) old[r] = (mine && r < nr) ? cp[(int64_t)r * ldc] : 0.0f;
+        }
+        uint32_t v[32];
+        tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) buf[lane * 33 + j] = __uint_as_float(v[j]);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            float out = buf[r * 33 + lane];
+            if (ab != 0) out = __fmul_rn(alpha, out);
+            if (ab == 2) out = __fadd_rn(out, __fmul_rn(beta, old[r]));
+            if (mine && r < nr) cp[(int64_t)r * ldc] = out;
+        }
+        __syncwarp();
+    }
+}
+
 // SPLIT > 1: the grid holds SPLIT CTAs per output tile, each over its own
 // contiguous range of K-blocks, which add their FP32 accumulators into C (set
 // to zero beforehand) instead of storing them.  c_tma: C is written through
@@ -114,7 +156,7 @@ template <int BN, int KB, int STAGES, int SPLIT>
 __global__ void __launch_bounds__(192, 1)
 prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, int c_tma, int M, int N, int K, float *__restrict__ C,
-                   int64_t ldc, uint32_t *flags, int pair_first)
+                   int64_t ldc, uint32_t *flags, int pair_first, float alpha, float beta, int ab)
 {
     using Cfg = F32Cfg<BN, KB, STAGES>;
     extern __shared__ uint8_t smem_raw[];
@@ -182,7 +224,8 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
         if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
-        else if (ok && SPLIT == 1) store_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
+        else if (ok && SPLIT == 1)
+            epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
         else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
@@ -228,7 +271,7 @@ template <int BN, int KB, int STAGES, int SPLIT>
 __global__ void __launch_bounds__(192, 1)
 prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmC, int c_tma, int M, int N, int K,
-                        float *__restrict__ C, int64_t ldc, uint32_t *flags)
+                        float *__restrict__ C, int64_t ldc, uint32_t *flags, float alpha, float beta, int ab)
 {
     using Cfg = F32PairCfg<BN, KB, STAGES>;
     extern __shared__ uint8_t smem_raw[];
@@ -312,7 +355,8 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
         if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
-        else if (ok && SPLIT == 1) store_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
+        else if (ok && SPLIT == 1)
+            epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
         else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
@@ -336,7 +380,7 @@ constexpr double kSplitCost = 0.95;
 template <int BN, int KB, int STAGES, int SPLIT = 1>
 cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp, int64_t ldcomp,
                     float *C, int64_t ldc, uint32_t *flags, cudaStream_t st, int64_t a_plane, int64_t b_plane,
-                    int pair_first = -1, int64_t pair_tiles = 0)
+                    float alpha, float beta, int ab, int pair_first = -1, int64_t pair_tiles = 0)
 {
     using Cfg = F32Cfg<BN, KB, STAGES>;
     CUtensorMap ta, tb;
@@ -346,7 +390,7 @@ cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const u
     // the epilogue writes (or adds) C through a C tensor map when one exists
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
-    const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
+    const int c_tma = ab == 0 && make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
     auto kern = prodsum_f32_kernel<BN, KB, STAGES, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
@@ -364,7 +408,8 @@ cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const u
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, C, ldc, flags, pair_first);
+    e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, C, ldc, flags, pair_first, alpha, beta,
+                           ab);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -372,7 +417,7 @@ cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const u
 template <int BN, int KB, int STAGES, int SPLIT>
 cudaError_t run_f32_pair(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp, int64_t ldcomp,
                          float *C, int64_t ldc, uint32_t *flags, cudaStream_t st, int64_t a_plane, int64_t b_plane,
-                         int64_t pair_tiles)
+                         float alpha, float beta, int ab, int64_t pair_tiles)
 {
     using Cfg = F32PairCfg<BN, KB, STAGES>;
     CUtensorMap ta, tb;
@@ -381,7 +426,7 @@ cudaError_t run_f32_pair(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, co
         return cudaErrorInvalidValue;
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
-    const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
+    const int c_tma = ab == 0 && make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
     auto kern = prodsum_f32_pair_kernel<BN, KB, STAGES, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
@@ -400,7 +445,7 @@ cudaError_t run_f32_pair(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, co
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, C, ldc, flags);
+    e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, C, ldc, flags, alpha, beta, ab);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -515,8 +560,9 @@ int f32_split_parts(int64_t M, int64_t N, int64_t K)
 
 cudaError_t launch_prodsum_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp,
                                int64_t ldcomp, float *C, int64_t ldc, uint32_t *flags, cudaStream_t st,
-                               int64_t a_plane, int64_t b_plane, bool c_zeroed)
+                               int64_t a_plane, int64_t b_plane, bool c_zeroed, float alpha, float beta, int ab)
 {
+    if (c_zeroed && ab != 0) return cudaErrorInvalidValue;
     int bn, parts;
     f32_tile_plan(M, N, K, c_zeroed, bn, parts);
     // 128 x 256 tiles run as 256 x 256 tiles on CTA pairs (64-wide K-blocks,
@@ -525,15 +571,20 @@ cudaError_t launch_prodsum_f32(int64_t M, int64_t N, int64_t K, const uint16_t *
     int64_t pairs, rest;
     if (bn == 256 && parts == 1 && f32_pair_plan(M, N, pairs, rest)) {
         cudaError_t e = run_f32_pair<256, 64, 2, 1>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane,
-                                                    pairs);
+                                                    alpha, beta, ab, pairs);
         if (e == cudaSuccess && rest > 0)
-            e = run_f32<128, 64, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, (int)pairs, rest);
+            e = run_f32<128, 64, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, alpha, beta, ab,
+                                    (int)pairs, rest);
         return e;
     }
-    if (parts == 2) return run_f32<128, 64, 2, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane);
-    if (bn == 128) return run_f32<128, 64, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane);
-    if (bn == 64) return run_f32<64, 64, 3>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane);
-    return run_f32<256, 32, 3>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane);
+    if (parts == 2) return run_f32<128, 64, 2, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, alpha,
+                                                       beta, ab);
+    if (bn == 128) return run_f32<128, 64, 2>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, alpha,
+                                                       beta, ab);
+    if (bn == 64) return run_f32<64, 64, 3>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, alpha,
+                                                       beta, ab);
+    return run_f32<256, 32, 3>(M, N, K, Ap, Bp, ldcomp, C, ldc, flags, st, a_plane, b_plane, alpha,
+                                                       beta, ab);
 }
 
 }  // namespace emu

@@ -277,6 +277,9 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // set-up above overlaps the end of the kernel that wrote the planes and levels
+    // (launched as its programmatic dependent)
+    griddep_wait();
 
     if (warp < Cfg::FIRST_DRAIN) {
       regs_dec<Cfg::REG_CTRL>();
@@ -862,13 +865,15 @@ cudaError_t run_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const 
     cfg.blockDim = dim3(Cfg::THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = PAIR ? 2 : 1;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = PAIR ? 1 : 0;
+    cfg.numAttrs = PAIR ? 2 : 1;
     e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, nprod, vA, vB, C, ldc, acc, flags, T,
                            ldt, wide_first);
     if (e != cudaSuccess) return e;

@@ -228,27 +228,39 @@ split_f32_transpose_kernel(const float *__restrict__ X, int64_t rows, int64_t co
                       &ws->flags);
 }
 
-// Both operands of an FP32 GEMM in one launch: blocks [0, nA) split A into
-// row-major planes (by rows on an ax x (nA / ax) grid when ax > 0, else by
-// 64 x 64 tiles), blocks [nA, nA + nB) split B into K-major planes, and
-// blocks from nA + nB on set the M x N result C to zero (a product-sum that
-// adds its K-parts into C needs it cleared).
+// One operand of a split of two: X as stored, the rows of its planes, its share
+// of the grid (n blocks) and how they walk it: transposed tiles, rows on an
+// ax x (n / ax) grid (ax > 0), or 64 x 64 row-major tiles.
+struct F32Operand {
+    const float *X;
+    int64_t rows, cols, ldx;
+    uint16_t *comps;
+    int64_t plane, n, ax;
+    bool transpose;
+};
+
+// Both operands of an FP32 GEMM in one launch: blocks [0, a.n) split A, the next
+// b.n split B, and the last nC set the M x N result C to zero (a product-sum
+// that adds its K-parts into C needs it cleared).
 __global__ void __launch_bounds__(kThreads)
-split_f32_gemm_kernel(const float *__restrict__ A, int64_t M, int64_t K, int64_t lda, const float *__restrict__ B,
-                      int64_t N, int64_t ldb, uint16_t *__restrict__ Ap, uint16_t *__restrict__ Bp, int64_t ldcomp,
-                      WsHeader *ws, int64_t ax, int64_t nA, int64_t nB, float *__restrict__ C, int64_t ldc, int64_t nC)
+split_f32_gemm_kernel(const __grid_constant__ F32Operand oa, const __grid_constant__ F32Operand ob, int64_t ldcomp,
+                      WsHeader *ws, float *__restrict__ C, int64_t M, int64_t N, int64_t ldc, int64_t nC)
 {
     __shared__ __align__(16) uint32_t sm[3][kTile][kTile / 2];
     // the product-sum launched after this kernel may start its set-up as soon
     // as every block of this one is running (it waits for all of it before
     // reading planes or C)
     griddep_launch_dependents();
+    const int64_t nA = oa.n, nB = ob.n;
     const int64_t b = blockIdx.x;
     if (b < nA + nB) {
+        const F32Operand &o = b < nA ? oa : ob;
+        const int64_t i = b < nA ? b : b - nA;
         const uint32_t amax =
-            b >= nA ? split_f32_transpose_body(B, K, N, ldb, Bp, ldcomp, N * ldcomp, ws, b - nA, nB, sm)
-            : ax > 0 ? split_f32_rows_body(A, M, K, lda, Ap, ldcomp, M * ldcomp, ws, b % ax, b / ax, nA / ax)
-                     : split_f32_rowtile_body(A, M, K, lda, Ap, ldcomp, M * ldcomp, b, nA);
+            o.transpose ? split_f32_transpose_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i, o.n, sm)
+            : o.ax > 0 ? split_f32_rows_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i % o.ax, i / o.ax,
+                                             o.n / o.ax)
+                       : split_f32_rowtile_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, i, o.n);
         // the flag word is cleared by the operation before this launch, which
         // may still be running when this kernel is its programmatic dependent
         griddep_wait();
@@ -291,37 +303,40 @@ cudaError_t launch_split_f32(const float *X, int64_t rows, int64_t cols, int64_t
     return cudaGetLastError();
 }
 
-// Both operands of an FP32 GEMM (A: M x K, B: K x N) into planes of row
-// pitch ldcomp laid out as the GEMM workspace holds them, in one launch; with
-// C non-null also C <- 0.
+// Both operands of an FP32 GEMM, op(A) (M x K) and op(B) (K x N), into planes of
+// row pitch ldcomp laid out as the GEMM workspace holds them, in one launch; with
+// C non-null also C <- 0.  ta / tb: the stored matrix is read transposed.
 cudaError_t launch_split_f32_gemm(const float *A, int64_t M, int64_t K, int64_t lda, const float *B, int64_t N,
                                   int64_t ldb, uint16_t *Ap, uint16_t *Bp, int64_t ldcomp, WsHeader *ws, float *C,
-                                  int64_t ldc, cudaStream_t st)
+                                  int64_t ldc, cudaStream_t st, bool ta, bool tb)
 {
     if (M == 0 || N == 0 || K == 0) return cudaSuccess;
-    // Operands of at most 256 tiles of 64 x 64 each: one block per tile, A by
+    F32Operand a = {A, ta ? K : M, ta ? M : K, lda, Ap, M * ldcomp, 0, 0, ta};
+    F32Operand b = {B, tb ? K : N, tb ? N : K, ldb, Bp, N * ldcomp, 0, 0, tb};
+    // Operands of at most 256 tiles of 64 x 64 each: one block per tile, rows by
     // tiles too, and at most 96 blocks clearing C, so that the launch is one
     // wave (608 blocks: four 256-thread blocks per SM at the kernel's 64
-    // registers) and its time one round trip to DRAM.  Larger operands: rows
-    // of A on 608 blocks, 608 blocks of B tiles (measured faster there).
-    const int64_t tiles_a = ((M + kTile - 1) / kTile) * ((K + kTile - 1) / kTile);
-    const int64_t tiles_b = ((K + kTile - 1) / kTile) * ((N + kTile - 1) / kTile);
-    const bool small = tiles_a <= 256 && tiles_b <= 256;
-    int64_t ax = 0, nA = tiles_a, nB = tiles_b, nC = 0;
-    if (small) {
-        nC = C ? (M < 96 ? M : 96) : 0;
-    } else {
-        ax = (K + 8 * kThreads - 1) / (8 * kThreads);
-        const int64_t want = (152 * 4 + ax - 1) / ax;
-        nA = ax * (M < want ? M : want);
-        nB = grid_for(tiles_b, 152 * 4);
-        nC = C ? (M < 152 ? M : 152) : 0;
+    // registers) and its time one round trip to DRAM.  Larger operands: 608
+    // blocks each, over rows or transposed tiles (measured faster there).
+    auto tiles = [](const F32Operand &o) { return ((o.rows + kTile - 1) / kTile) * ((o.cols + kTile - 1) / kTile); };
+    const bool small = tiles(a) <= 256 && tiles(b) <= 256;
+    for (F32Operand *o : {&a, &b}) {
+        if (small) {
+            o->n = tiles(*o);
+        } else if (o->transpose) {
+            o->n = grid_for(tiles(*o), 152 * 4);
+        } else {
+            o->ax = (o->cols + 8 * kThreads - 1) / (8 * kThreads);
+            const int64_t want = (152 * 4 + o->ax - 1) / o->ax;
+            o->n = o->ax * (o->rows < want ? o->rows : want);
+        }
     }
+    const int64_t most = small ? 96 : 152, nC = C ? (M < most ? M : most) : 0;
     cudaError_t e;
     // a programmatic dependent of the clearing of the workspace header, which
     // only its flag publication waits for
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nA + nB + nC));
+    cfg.gridDim = dim3((unsigned)(a.n + b.n + nC));
     cfg.blockDim = dim3(kThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -329,8 +344,7 @@ cudaError_t launch_split_f32_gemm(const float *A, int64_t M, int64_t K, int64_t 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, split_f32_gemm_kernel, A, M, K, lda, B, N, ldb, Ap, Bp, ldcomp, ws, ax, nA, nB, C,
-                           ldc, nC);
+    e = cudaLaunchKernelEx(&cfg, split_f32_gemm_kernel, a, b, ldcomp, ws, C, M, N, ldc, nC);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -191,6 +191,173 @@ f64_spec_transpose_kernel(const double *__restrict__ X, int64_t rows, int64_t co
     f64_spec_transpose_body<NLEV>(X, rows, cols, ldx, comps, ldcomp, plane, ws, slot, blockIdx.x, gridDim.x, smw, red);
 }
 
+// Row-major planes of an operand too small for the row pass to fill its blocks:
+// a 64 x 64 tile per step, 16 threads to a row of it (four entries each).
+// Block bid of nblk; red: 5 * kThreads / 32 words of shared memory.
+template <int NLEV>
+__device__ __forceinline__ void f64_spec_tile_body(const double *__restrict__ X, int64_t rows, int64_t cols, int64_t ldx,
+                                                   uint16_t *__restrict__ comps, int64_t ldcomp, int64_t plane,
+                                                   WsHeader *ws, int slot, int64_t bid, int64_t nblk, uint32_t *red)
+{
+    const int v0 = spec_v0(ws, slot);
+    const bool fast = v0 >= -78;
+    float P[3] = {};
+    if (fast) spec_units(v0 - 50, P);
+    const bool vin = ((ldx & 1) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0);
+    const bool vout = ((ldcomp & 3) == 0) && ((plane & 3) == 0) && ((reinterpret_cast<uintptr_t>(comps) & 7u) == 0);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int64_t tiles_r = (rows + kTile - 1) / kTile, tiles_c = (cols + kTile - 1) / kTile;
+    SpecState st;
+    for (int64_t t = bid; t < tiles_r * tiles_c; t += nblk) {
+        const int64_t j0 = (t % tiles_c) * kTile + 4 * tx;
+        const bool full = j0 + 4 <= cols;
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p) {
+            const int64_t i = (t / tiles_c) * kTile + ty + 16 * p;
+            if (i >= rows || j0 >= cols) continue;
+            const double *src = X + i * ldx + j0;
+            double x[4];
+            if (vin && full) {
+                const double2 a = reinterpret_cast<const double2 *>(src)[0], c = reinterpret_cast<const double2 *>(src)[1];
+                x[0] = a.x; x[1] = a.y; x[2] = c.x; x[3] = c.y;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[e] = (j0 + e < cols) ? src[e] : 0.0;
+            }
+            uint32_t w[NLEV][2];
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {
+                uint32_t sa[6], sb[6];
+                spec_element<NLEV>(x[e], v0, fast, P, sa, st);
+                spec_element<NLEV>(x[e + 1], v0, fast, P, sb, st);
+#pragma unroll
+                for (int r = 0; r < NLEV; ++r) w[r][e >> 1] = pack2(sa[r], sb[r]);
+            }
+            uint16_t *dst = comps + i * ldcomp + j0;
+#pragma unroll
+            for (int r = 0; r < NLEV; ++r) {
+                if (vout && full) {
+                    *reinterpret_cast<uint2 *>(dst + r * plane) = make_uint2(w[r][0], w[r][1]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (j0 + e < cols) dst[r * plane + e] = (uint16_t)(w[r][e >> 1] >> (16 * (e & 1)));
+                }
+            }
+        }
+    }
+    spec_publish(st, v0, ws, slot, red);
+}
+
+// One operand of a split of two: X as stored, its planes, whether they are
+// written transposed, and where its levels go.
+struct SplitOperand {
+    const double *X;
+    int64_t rows, cols, ldx;
+    uint16_t *comps;
+    int64_t plane;
+    int32_t *v_out;
+    bool transpose;
+};
+
+// The literal passes of one operand whose speculative levels failed from level
+// ff on, as f64_fix_kernel runs them (every block of a cooperative launch).
+__device__ __noinline__ void fix_operand(const SplitOperand &o, int64_t ldcomp, WsHeader *ws, int slot, int ff,
+                                         const int (&v)[6], int nlev, unsigned long long *red, uint16_t *smdyn)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        for (int r = 0; r < 6; ++r) ws->v[slot][r] = v[r];
+        ws->fix_from[slot] = ff;
+    }
+    grid_sync(ws, slot);
+    f64_max_pass<1>(o.X, o.rows, o.cols, o.ldx, ws, slot, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, slot);
+    f64_max_pass<2>(o.X, o.rows, o.cols, o.ldx, ws, slot, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, slot);
+    f64_max_pass<3>(o.X, o.rows, o.cols, o.ldx, ws, slot, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, slot);
+    f64_max_pass<4>(o.X, o.rows, o.cols, o.ldx, ws, slot, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, slot);
+    f64_max_pass<5>(o.X, o.rows, o.cols, o.ldx, ws, slot, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, slot);
+    if (o.transpose)
+        split_tile_pass<double, 2, true>(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, slot, nullptr,
+                                         nullptr, blockIdx.x, gridDim.x, smdyn);
+    else
+        split_tile_pass<double, 2, false>(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, slot, nullptr,
+                                          nullptr, blockIdx.x, gridDim.x, smdyn);
+    grid_sync(ws, slot);
+    if (blockIdx.x == 0 && threadIdx.x == 0) f64_finalize(ws, slot, o.v_out, nlev);
+}
+
+// After the speculative passes of both operands: every block checks both; the
+// usual case publishes the levels and ends, no block waiting on another.
+__device__ __forceinline__ void verify_and_fix(const SplitOperand &a, const SplitOperand &b, int64_t ldcomp, WsHeader *ws,
+                                               int nlev, unsigned long long *red, uint16_t *smdyn)
+{
+#pragma unroll 1
+    for (int slot = 0; slot < 2; ++slot) {
+        int v[6];
+        const int ff = f64_verify_levels(ws, slot, v, nlev);
+        const SplitOperand &o = slot ? b : a;
+        if (ff == 6) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                for (int r = 0; r < 6; ++r) ws->v[slot][r] = v[r];
+                ws->fix_from[slot] = 6;
+                f64_finalize(ws, slot, o.v_out, nlev);
+            }
+        } else {
+            fix_operand(o, ldcomp, ws, slot, ff, v, nlev, red, smdyn);
+        }
+    }
+}
+
+// The verifier of both operands as one cooperative launch.
+__global__ void __launch_bounds__(kThreads)
+f64_fix_pair_kernel(const __grid_constant__ SplitOperand a, const __grid_constant__ SplitOperand b, int64_t ldcomp,
+                    WsHeader *ws, int nlev)
+{
+    extern __shared__ __align__(16) uint16_t smdyn[];
+    __shared__ unsigned long long red[kThreads / 32];
+    griddep_launch_dependents();
+    verify_and_fix(a, b, ldcomp, ws, nlev, red, smdyn);
+}
+
+// The whole split of two small operands in one cooperative launch: level-0
+// maxima, grid barrier, speculative pass by tiles, grid barrier, verifier.  Five
+// launches and their gaps took 28 us for operands of 256 x 256, whose entries
+// are read and written in well under one.
+template <int NLEV>
+__global__ void __launch_bounds__(kThreads)
+f64_split_small_kernel(const __grid_constant__ SplitOperand a, const __grid_constant__ SplitOperand b, int64_t ldcomp,
+                       WsHeader *ws)
+{
+    extern __shared__ __align__(16) uint32_t smw[];
+    __shared__ unsigned long long red[5 * (kThreads / 32)];
+    uint32_t *red32 = reinterpret_cast<uint32_t *>(red);
+    griddep_launch_dependents();
+    f64_max_pass<0>(a.X, a.rows, a.cols, a.ldx, ws, 0, blockIdx.x, gridDim.x, red);
+    f64_max_pass<0>(b.X, b.rows, b.cols, b.ldx, ws, 1, blockIdx.x, gridDim.x, red);
+    grid_sync(ws, 0);
+    // B's tiles go on where A's end, so that a block has tiles of one operand only while
+    // there are blocks enough
+    const int64_t ta = ((a.rows + kTile - 1) / kTile) * ((a.cols + kTile - 1) / kTile);
+    const int64_t bid_b = (blockIdx.x + gridDim.x - ta % gridDim.x) % gridDim.x;
+#pragma unroll 1
+    for (int slot = 0; slot < 2; ++slot) {
+        const SplitOperand &o = slot ? b : a;
+        const int64_t bid = slot ? bid_b : blockIdx.x;
+        if (o.transpose)
+            f64_spec_transpose_body<NLEV>(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, slot, bid, gridDim.x,
+                                          smw, red32);
+        else
+            f64_spec_tile_body<NLEV>(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, slot, bid, gridDim.x, red32);
+        __syncthreads();                                  // red is reused
+    }
+    grid_sync(ws, 1);
+    verify_and_fix(a, b, ldcomp, ws, NLEV, red, reinterpret_cast<uint16_t *>(smw));
+}
+
 // Block b of a launch that holds nA blocks of one kind and nB of another:
 // the first 2 min(nA, nB) blocks alternate between the kinds (blocks are
 // dispatched roughly in index order, so both kinds run side by side), the
@@ -206,14 +373,15 @@ __device__ __forceinline__ int64_t pair_block(int64_t b, int64_t nA, int64_t nB,
 // The level-0 maxima of both operands of an FP64 GEMM in one launch: nA
 // blocks on A (header slot 0) and nB on B (slot 1), interleaved.
 __global__ void __launch_bounds__(kThreads)
-f64_max_gemm_kernel(const double *__restrict__ A, int64_t M, int64_t K, int64_t lda, const double *__restrict__ B,
-                    int64_t N, int64_t ldb, WsHeader *ws, int64_t nA, int64_t nB)
+f64_max_gemm_kernel(const double *__restrict__ A, int64_t rows_a, int64_t cols_a, int64_t lda,
+                    const double *__restrict__ B, int64_t rows_b, int64_t cols_b, int64_t ldb, WsHeader *ws, int64_t nA,
+                    int64_t nB)
 {
     __shared__ unsigned long long red[kThreads / 32];
     bool is_a;
     const int64_t i = pair_block(blockIdx.x, nA, nB, is_a);
-    if (is_a) f64_max_pass<0>(A, M, K, lda, ws, 0, i, nA, red);
-    else f64_max_pass<0>(B, K, N, ldb, ws, 1, i, nB, red);
+    if (is_a) f64_max_pass<0>(A, rows_a, cols_a, lda, ws, 0, i, nA, red);
+    else f64_max_pass<0>(B, rows_b, cols_b, ldb, ws, 1, i, nB, red);
 }
 
 // The fused speculative pass for slices 0 .. NLEV-1.
@@ -269,55 +437,111 @@ cudaError_t launch_split_f64(const double *X, int64_t rows, int64_t cols, int64_
 }
 
 
-// Both operands of an FP64 GEMM (A: M x K into row-major planes, B: K x N
-// into K-major planes, row pitch ldcomp), with the level maxima of A and B in
-// one launch; the speculative passes and verifiers stay one launch per
-// operand.  Results are those of launch_split_f64 on A, then B.
+namespace {
+
+// Cooperative launch of `kern` with as many blocks as fit on the device at once,
+// at most `want` (the limit is found once per device and kernel).
+template <typename... Args>
+cudaError_t launch_cooperative(void (*kern)(Args...), int (&fits)[64], int64_t want, cudaStream_t st, Args... values)
+{
+    const size_t sm = smem_bytes(6) > kSpecTransposeSmem ? smem_bytes(6) : kSpecTransposeSmem;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    int most = fits[dev];
+    if (most == 0) {
+        int sms = 0, per = 0;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, sm);
+        if (e != cudaSuccess) return e;
+        most = per * sms < 152 * 8 ? per * sms : 152 * 8;
+        if (most < 1) return cudaErrorInvalidConfiguration;
+        fits[dev] = most;
+    }
+    void *args[] = {(void *)&values...};
+    return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)(want < most ? want : most)), dim3(kThreads),
+                                       args, sm, st);
+}
+
+template <int NLEV>
+cudaError_t launch_small(const SplitOperand &a, const SplitOperand &b, int64_t ldcomp, int64_t tiles, WsHeader *ws,
+                         cudaStream_t st)
+{
+    static int fits[64] = {};
+    return launch_cooperative(f64_split_small_kernel<NLEV>, fits, tiles < 152 ? 152 : tiles, st, a, b, ldcomp, ws);
+}
+
+template <int NLEV>
+cudaError_t launch_spec_pair(const SplitOperand &a, const SplitOperand &b, int64_t ldcomp, WsHeader *ws, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    for (int slot = 0; slot < 2 && e == cudaSuccess; ++slot) {
+        const SplitOperand &o = slot ? b : a;
+        const int gt = grid_for(((o.rows + kTile - 1) / kTile) * ((o.cols + kTile - 1) / kTile), 152 * 8);
+        e = launch_spec<NLEV>(o.X, o.rows, o.cols, o.ldx, o.transpose, o.comps, ldcomp, o.plane, ws, slot, gt, st);
+    }
+    return e;
+}
+
+// Operands of together at most this many entries are split in one launch.
+constexpr int64_t kSmallSplit = (int64_t)1 << 22;
+
+}  // namespace
+
+// Both operands of an FP64 GEMM: op(A) (M x K) into planes [s][M][ldcomp] and
+// op(B) (K x N) into planes [s][N][ldcomp]; ta / tb: the stored matrix is read
+// transposed to become the planes' rows (A stored K x M; B stored K x N).
+// Small operands take one launch; larger ones the level maxima of both in one
+// launch, a speculative pass each and the verifier of both.  Results are those
+// of launch_split_f64 on A, then B.
 cudaError_t launch_split_f64_gemm(const double *A, int64_t M, int64_t K, int64_t lda, const double *B, int64_t N,
                                   int64_t ldb, uint16_t *Ap, uint16_t *Bp, int64_t ldcomp, int32_t *vA_out,
-                                  int32_t *vB_out, WsHeader *ws, cudaStream_t st, int nlev)
+                                  int32_t *vB_out, WsHeader *ws, cudaStream_t st, int nlev, bool ta, bool tb)
 {
     if (nlev < 3 || nlev > 6) return cudaErrorInvalidValue;
+    const SplitOperand a = {A, ta ? K : M, ta ? M : K, lda, Ap, M * ldcomp, vA_out, ta};
+    const SplitOperand b = {B, tb ? K : N, tb ? N : K, ldb, Bp, N * ldcomp, vB_out, tb};
     if (M == 0 || N == 0 || K == 0) {
-        cudaError_t e = launch_split_f64(A, M, K, lda, false, Ap, ldcomp, vA_out, ws, 0, st, nlev);
-        if (e == cudaSuccess) e = launch_split_f64(B, K, N, ldb, true, Bp, ldcomp, vB_out, ws, 1, st, nlev);
+        cudaError_t e = launch_split_f64(A, a.rows, a.cols, lda, ta, Ap, ldcomp, vA_out, ws, 0, st, nlev);
+        if (e == cudaSuccess) e = launch_split_f64(B, b.rows, b.cols, ldb, tb, Bp, ldcomp, vB_out, ws, 1, st, nlev);
         return e;
     }
+    if ((M + N) * K <= kSmallSplit) {
+        const int64_t tiles = ((M + kTile - 1) / kTile + (N + kTile - 1) / kTile) * ((K + kTile - 1) / kTile);
+        switch (nlev) {
+        case 3: return launch_small<3>(a, b, ldcomp, tiles, ws, st);
+        case 4: return launch_small<4>(a, b, ldcomp, tiles, ws, st);
+        case 5: return launch_small<5>(a, b, ldcomp, tiles, ws, st);
+        default: return launch_small<6>(a, b, ldcomp, tiles, ws, st);
+        }
+    }
     // level-0 maxima: blocks shared in proportion to the entries, at most 152 x 8 in all
-    const int64_t segA = M * ((K + 4 * kThreads - 1) / (4 * kThreads)), segB = K * ((N + 4 * kThreads - 1) / (4 * kThreads));
+    const int64_t segA = a.rows * ((a.cols + 4 * kThreads - 1) / (4 * kThreads));
+    const int64_t segB = b.rows * ((b.cols + 4 * kThreads - 1) / (4 * kThreads));
     const double fa = (double)(M * K) / (double)(M * K + K * N);
     int64_t nA = (int64_t)(152 * 8 * fa + 0.5), nB = 152 * 8 - nA;
     nA = nA < 1 ? 1 : (nA > segA ? segA : nA);
     nB = nB < 1 ? 1 : (nB > segB ? segB : nB);
-    f64_max_gemm_kernel<<<(unsigned)(nA + nB), kThreads, 0, st>>>(A, M, K, lda, B, N, ldb, ws, nA, nB);
+    f64_max_gemm_kernel<<<(unsigned)(nA + nB), kThreads, 0, st>>>(A, a.rows, a.cols, lda, B, b.rows, b.cols, ldb, ws, nA,
+                                                                  nB);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the speculative passes stay one launch per operand: in one launch the
     // row blocks would reserve the transposed blocks' shared memory (measured
     // 15-25 % slower)
-    const int gB = grid_for(((K + kTile - 1) / kTile) * ((N + kTile - 1) / kTile), 152 * 8);
     switch (nlev) {
-    case 3:
-        e = launch_spec<3>(A, M, K, lda, false, Ap, ldcomp, M * ldcomp, ws, 0, 0, st);
-        if (e == cudaSuccess) e = launch_spec<3>(B, K, N, ldb, true, Bp, ldcomp, N * ldcomp, ws, 1, gB, st);
-        break;
-    case 4:
-        e = launch_spec<4>(A, M, K, lda, false, Ap, ldcomp, M * ldcomp, ws, 0, 0, st);
-        if (e == cudaSuccess) e = launch_spec<4>(B, K, N, ldb, true, Bp, ldcomp, N * ldcomp, ws, 1, gB, st);
-        break;
-    case 5:
-        e = launch_spec<5>(A, M, K, lda, false, Ap, ldcomp, M * ldcomp, ws, 0, 0, st);
-        if (e == cudaSuccess) e = launch_spec<5>(B, K, N, ldb, true, Bp, ldcomp, N * ldcomp, ws, 1, gB, st);
-        break;
-    default:
-        e = launch_spec<6>(A, M, K, lda, false, Ap, ldcomp, M * ldcomp, ws, 0, 0, st);
-        if (e == cudaSuccess) e = launch_spec<6>(B, K, N, ldb, true, Bp, ldcomp, N * ldcomp, ws, 1, gB, st);
-        break;
+    case 3: e = launch_spec_pair<3>(a, b, ldcomp, ws, st); break;
+    case 4: e = launch_spec_pair<4>(a, b, ldcomp, ws, st); break;
+    case 5: e = launch_spec_pair<5>(a, b, ldcomp, ws, st); break;
+    default: e = launch_spec_pair<6>(a, b, ldcomp, ws, st); break;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_f64_fix(A, M, K, lda, false, Ap, ldcomp, M * ldcomp, ws, 0, vA_out, st, nlev);
-    if (e == cudaSuccess) e = launch_f64_fix(B, K, N, ldb, true, Bp, ldcomp, N * ldcomp, ws, 1, vB_out, st, nlev);
-    return e;
+    if (e != cudaSuccess) return e;
+    static int fits[64] = {};
+    return launch_cooperative(f64_fix_pair_kernel, fits, (int64_t)152 * 8, st, a, b, ldcomp, ws, nlev);
 }
 
 }  // namespace emu
