@@ -116,8 +116,9 @@ int f64_tile_columns(int64_t M, int64_t N);
 // in raster order of 128 x 256, or with pair of 256 x 256 on clusters of two
 // CTAs (launch_prodsum_f64_wide); of 128 x cols, cols = 128 or 64, or with pair
 // of 256 x 128, with wide_first >= 0 `tiles` halves of the 256 x 256 tiles from
-// raster index wide_first on (launch_prodsum_f64_narrow).  acc: f64_acc_bytes(M, N)
-// bytes.
+// raster index wide_first on (launch_prodsum_f64_narrow).  duo: two CTAs share
+// each 128-row tile's products (levels per matrix, no tail).  acc:
+// f64_acc_bytes(M, N) bytes.
 cudaError_t launch_prodsum_f64_wide(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp,
                                      int64_t ldcomp, const int32_t *vA, const int32_t *vB, int nprod, double *C,
                                      int64_t ldc, double *acc, uint32_t *flags, cudaStream_t st, int64_t a_plane,
@@ -126,7 +127,7 @@ cudaError_t launch_prodsum_f64_narrow(int64_t M, int64_t N, int64_t K, const uin
                                      int64_t ldcomp, const int32_t *vA, const int32_t *vB, int nprod, double *C,
                                      int64_t ldc, double *acc, uint32_t *flags, cudaStream_t st, int64_t a_plane,
                                      bool rowcol, const float *T, int64_t ldt, int cols, bool pair, int64_t tiles,
-                                      int wide_first);
+                                      int wide_first, bool duo);
 
 // Bytes of the FP64 product-sum's accumulator, enough for either tile shape:
 // one FP64 tile of 128 x 128 (narrow kernel) or 128 x 256 (wide kernel) per

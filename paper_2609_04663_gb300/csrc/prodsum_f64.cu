@@ -108,14 +108,17 @@ cudaError_t launch_prodsum_f64(int64_t M, int64_t N, int64_t K, const uint16_t *
                                bool rowcol, const float *T, int64_t ldt)
 {
     const F64Plan p = f64_plan(M, N);
+    // 128-row tiles on at most half of the SMs: two CTAs per tile, each with half of the
+    // first ten products (any K that diag_exact lets through)
+    const bool duo = p.cols < 256 && p.rows == 128 && !rowcol && !T && vA && 2 * p.tiles <= device_sms() && K <= 8097;
     if (p.cols < 256)
         return launch_prodsum_f64_narrow(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
-                                         rowcol, T, ldt, p.cols, p.rows == 256, p.tiles, -1);
+                                         rowcol, T, ldt, p.cols, p.rows == 256, p.tiles, -1, duo);
     cudaError_t e = launch_prodsum_f64_wide(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
                                             rowcol, T, ldt, p.rows == 256, p.tiles);
     if (e != cudaSuccess || p.rest == 0) return e;
     return launch_prodsum_f64_narrow(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane, rowcol, T,
-                                     ldt, 128, true, p.rest, (int)p.tiles);
+                                     ldt, 128, true, p.rest, (int)p.tiles, false);
 }
 
 }  // namespace emu

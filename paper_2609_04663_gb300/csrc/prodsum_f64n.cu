@@ -9,16 +9,16 @@ cudaError_t launch_prodsum_f64_narrow(int64_t M, int64_t N, int64_t K, const uin
                                      int64_t ldcomp, const int32_t *vA, const int32_t *vB, int nprod, double *C,
                                      int64_t ldc, double *acc, uint32_t *flags, cudaStream_t st, int64_t a_plane,
                                      bool rowcol, const float *T, int64_t ldt, int cols, bool pair, int64_t tiles,
-                                      int wide_first)
+                                      int wide_first, bool duo)
 {
     if (f64_diagonals(nprod) == 0) return cudaErrorInvalidValue;
     if (pair)
         return dispatch_f64w<128, true>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane, rowcol, T,
                                         ldt, tiles, wide_first);
     return cols == 128 ? dispatch_f64w<128, false>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st,
-                                                   a_plane, rowcol, T, ldt, tiles, wide_first)
+                                                   a_plane, rowcol, T, ldt, tiles, wide_first, duo)
                        : dispatch_f64w<64, false>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st,
-                                                  a_plane, rowcol, T, ldt, tiles, wide_first);
+                                                  a_plane, rowcol, T, ldt, tiles, wide_first, duo);
 }
 
 }  // namespace emu

@@ -97,7 +97,7 @@ struct F64WCfgT {
     static constexpr int CODE_OFF = STAGES * STAGE;
     static constexpr int LVL_OFF = CODE_OFF + kBM * BN;
     static constexpr int BAR_OFF = LVL_OFF + BN * 4;
-    static constexpr int NBARS = 2 * STAGES + 2 * NBUF + 1;
+    static constexpr int NBARS = 2 * STAGES + 2 * NBUF + 3;   // done, and two between the CTAs of a duo
     static constexpr int SMEM = BAR_OFF + 256 + 1024;
     // Register split: the launch reserves 384 x 168 = 128 x 40 (control) + 256 x
     // 232 (drain), or 640 x 96 = 128 x 32 + 512 x 112.
@@ -178,6 +178,43 @@ __device__ __forceinline__ int level_gap(const int32_t *v, int64_t stride, int d
     return w;
 }
 
+// Levels per matrix in steps of 8 whose units, with the rounding constants (2^-25 u
+// to 2^(23 + kMaxRoundBits) u), are normal; e0 = vA_0 + vB_0 then.
+__device__ __forceinline__ bool matrix_lock(const int32_t *vA, const int32_t *vB, int d, int &e0)
+{
+    if (!vA || vA[0] == kZeroLevel || vB[0] == kZeroLevel) return false;
+    e0 = vA[0] + vB[0];
+    return level_gap(vA, 1, d, vA[0]) == 0 && level_gap(vB, 1, d, vB[0]) == 0 && e0 <= 100 && e0 + 8 - 8 * (d - 1) >= -76;
+}
+
+// Number of diagonals of nprod products.
+__device__ __forceinline__ int diagonals_of(int nprod) { return nprod == 6 ? 3 : nprod == 10 ? 4 : nprod == 15 ? 5 : 6; }
+
+// CTA of a duo that computes product q: whole diagonals each, 3 + 3 of 6 products,
+// 5 + 5 of the first 10, and the first CTA any later ones.
+__device__ __forceinline__ uint32_t duo_owner(int q, int nprod)
+{
+    return nprod == 6 ? (q < 3 ? 0u : 1u) : (q == 0 || q >= 6 ? 0u : 1u);
+}
+
+// Every lane's global writes and reductions so far become visible to the other
+// CTA of the duo when its wait on `bar` (count: the drain warps) completes.
+__device__ __forceinline__ void signal_duo(uint32_t bar, uint32_t rank)
+{
+    __threadfence();
+    __syncwarp();
+    if (lane_id() == 0)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(peer_addr(bar, rank ^ 1u))
+                     : "memory");
+    __syncwarp();
+}
+__device__ __forceinline__ bool wait_duo(uint32_t bar, uint32_t *flags)
+{
+    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, 0, flags));
+    __threadfence();
+    return ok;
+}
+
 // Code byte of an element while its running sum is rounded to multiples of g =
 // 2^n u: bits 0-6 hold n + 48 (kCodeKeep where g <= u: nothing to round;
 // kCodeEach: reduced after every product), bit 7 says that the sum started
@@ -208,17 +245,25 @@ __device__ __forceinline__ float start_of(uint32_t code, uint32_t bound_bits)
 }
 
 // TAIL: add the merged tail T (an M x N FP32 matrix) once after the last product.
+// vA, vB and T are written by the kernels before this one, which may still run when
+// it starts: not __restrict__, so that no load of them moves above griddep_wait.
 // wide_first >= 0 (pairs with BN = 128): this launch takes the 256 x 128 halves
 // of the 256 x 256 tiles from raster index wide_first on.
-template <int BN, bool ROWCOL, bool TAIL, bool PAIR>
+// DUO: a cluster of two CTAs shares a tile's products.  While every addition up to
+// the fourth diagonal is exact (diag_exact; levels in steps of 8), sums may reach
+// the accumulator in any order, so the second CTA takes half of the first six or
+// ten products; the first stores product 0 before the second reduces, the later
+// diagonals (first CTA) wait for both halves, and each CTA writes half of the
+// tile to C.  Otherwise the first CTA does everything.
+template <int BN, bool ROWCOL, bool TAIL, bool PAIR, bool DUO>
 __global__ void __launch_bounds__(F64WCfgT<BN, PAIR>::THREADS, 1)
 prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, int c_tma, int M, int N, int K, int nprod,
-                    const int32_t *__restrict__ vA, const int32_t *__restrict__ vB, double *__restrict__ C,
-                    int64_t ldc, double *__restrict__ acc, uint32_t *flags, const float *__restrict__ T, int64_t ldt,
-                    int wide_first)
+                    const int32_t *vA, const int32_t *vB, double *__restrict__ C, int64_t ldc, double *__restrict__ acc,
+                    uint32_t *flags, const float *T, int64_t ldt, int wide_first)
 {
     using Cfg = F64WCfgT<BN, PAIR>;
+    static_assert(!DUO || (!PAIR && !ROWCOL && !TAIL), "duos: one CTA per MMA, levels per matrix, no tail");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -230,7 +275,8 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     LevelSummary *lsum = reinterpret_cast<LevelSummary *>(base_ptr + Cfg::BAR_OFF + 8 * Cfg::NBARS + 8);
 
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    const uint32_t rank = PAIR ? cluster_rank() : 0u;
+    const uint32_t rank = PAIR || DUO ? cluster_rank() : 0u;
+    const uint32_t duo_first = done_bar + 8u, duo_done = done_bar + 16u;   // product 0 stored; the other CTA's sums reduced
     const int tiles_n = (N + BN - 1) / BN;
     int tm, tn;
     if constexpr (PAIR) {                             // the pair's 256 rows: this CTA takes half `rank`
@@ -247,7 +293,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
         tm = 2 * tp + (int)rank;
     } else {
-        tile_coords(blockIdx.x, (M + kBM - 1) / kBM, tiles_n, tm, tn);
+        tile_coords((int)(DUO ? blockIdx.x >> 1 : blockIdx.x), (M + kBM - 1) / kBM, tiles_n, tm, tn);
     }
     const int m0 = tm * kBM, n0 = tn * BN;
     const int nch = (K + kKChunk - 1) / kKChunk;
@@ -261,6 +307,8 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             mbar_init(tempty0 + 8u * b, (PAIR ? 2 : 1) * Cfg::DRAIN_WARPS);
         }
         mbar_init(done_bar, 1);
+        mbar_init(duo_first, Cfg::DRAIN_WARPS);
+        mbar_init(duo_done, Cfg::DRAIN_WARPS);
         fence_mbar_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
@@ -273,6 +321,10 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     } else {
         if (warp == 1) { tmem_alloc(smem_u32((const void *)tmem_slot), 512); tmem_relinquish(); }
     }
+    if constexpr (DUO) {
+        __syncthreads();
+        cluster_sync();                               // both CTAs' barriers initialised
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -280,6 +332,12 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     // set-up above overlaps the end of the kernel that wrote the planes and levels
     // (launched as its programmatic dependent)
     griddep_wait();
+    int e0 = 0;
+    bool lock = false;
+    if constexpr (!ROWCOL) lock = matrix_lock(vA, vB, diagonals_of(nprod), e0);
+    const bool duo = DUO && lock && diag_exact(K, min(3, diagonals_of(nprod) - 1));
+    // whether this CTA computes product q
+    auto mine_q = [&](int q) { return !DUO || (duo ? duo_owner(q, nprod) == rank : rank == 0); };
 
     if (warp < Cfg::FIRST_DRAIN) {
       regs_dec<Cfg::REG_CTRL>();
@@ -289,6 +347,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         uint32_t ph = 0;
         bool ok = true;
         for (int q = 0; q < nprod && ok; ++q) {
+            if (!mine_q(q)) continue;
             const int ia = kDiag[q][0], jb = kDiag[q][1];
             for (int c = 0; c < nch && ok; ++c) {
                 const int kbs = min(kKChunk / Cfg::KB, (K - c * kKChunk + Cfg::KB - 1) / Cfg::KB);
@@ -312,7 +371,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
         }
         if (!ok) {
-            if (rank == 0) {
+            if (!PAIR || rank == 0) {
                 drain_inflight(full0, Cfg::STAGES, L, flags);
             } else {
                 // the peer's copies complete on the leader's barriers, which it
@@ -321,7 +380,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 while (globaltimer_ns() - t0 < 200000ull) {}
             }
         }
-      } else if (warp == 1 && rank == 0) {
+      } else if (warp == 1 && (!PAIR || rank == 0)) {
         // ---------------- MMA issuer (a pair's leader): one chunk partial into buffer t % NBUF.
         // The whole warp walks the loop (waits decided by vote), one elected lane
         // issues: control flow and operands are then uniform, and the descriptors
@@ -332,7 +391,9 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         int s = 0, b = 0, c = 0;
         uint32_t ph = 0, tph = 0;
         bool ok = true;
-        for (int t = 0; t < nprod * nch && ok; ++t) {
+        int nmine = 0;                                // products of this CTA
+        for (int q = 0; q < nprod; ++q) nmine += mine_q(q) ? 1 : 0;
+        for (int t = 0; t < nmine * nch && ok; ++t) {
             const int kbs = min(kKChunk / Cfg::KB, (K - c * kKChunk + Cfg::KB - 1) / Cfg::KB);
             if (!(ok = __all_sync(0xFFFFFFFFu, mbar_wait(tempty0 + 8u * b, tph ^ 1u, flags)))) break;
             tc_fence_after();
@@ -386,15 +447,14 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // accumulator's stripes: its threads touch neither the accumulator nor C
         const bool live = !PAIR || row < M;
         // the low words live in one half of this thread's C words until their group is reduced
-        float *lrow = reinterpret_cast<float *>(crow);
+        float *lrow = reinterpret_cast<float *>(crow) + (DUO ? rank : 0u);
         uint32_t *codes = reinterpret_cast<uint32_t *>(base_ptr + Cfg::CODE_OFF) + dt;   // word w at w * DRAIN_THREADS
         int *lvl = reinterpret_cast<int *>(base_ptr + Cfg::LVL_OFF) + cq * Cfg::COLS;
 
         // Levels.  lock: the units of a diagonal's products agree, and they and the rounding
-        // constants (2^-25 u to 2^(23 + kMaxRoundBits) u) are normal.
-        const int d = nprod == 6 ? 3 : nprod == 10 ? 4 : nprod == 15 ? 5 : 6;
-        int e0 = 0, row_e = 0, row_gap = 0, lvl_min = 0;
-        bool lock = false;
+        // constants are normal (matrix_lock).
+        const int d = diagonals_of(nprod);
+        int row_e = 0, row_gap = 0, lvl_min = 0;
         if constexpr (ROWCOL) {
             // lvl[column]: (v_0 - gap + 68) << 23, so that adding (v_0 - gap + 67) << 23 of the
             // row gives the bits of the FP32 bound 2^24 u (integer order is the order of
@@ -429,10 +489,6 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             lvl_min = 0x7FFFFFFF;
 #pragma unroll 4
             for (int j = 0; j < Cfg::COLS; ++j) lvl_min = min(lvl_min, lvl[j]);
-        } else if (vA && vA[0] != kZeroLevel && vB[0] != kZeroLevel) {
-            e0 = vA[0] + vB[0];
-            lock = level_gap(vA, 1, d, vA[0]) == 0 && level_gap(vB, 1, d, vB[0]) == 0 && e0 <= 100 &&
-                   e0 + 8 - 8 * (d - 1) >= -76;
         }
         const int group = lock ? max(1, kGroupChunks / nch) : 1;          // most products in a group
 
@@ -447,7 +503,18 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         bool each = false;                                    // some element is reduced after every product
         int diag = 0, in_diag = 0, in_group = 0;              // product q: diagonal, place in it and in its group
         bool ok = true;
+        int t0 = 0;                                           // chunk partials before product q
+        bool first_in = !duo || rank == 0, others_in = !duo;  // what this CTA has waited for
         for (int q = 0; q < nprod && ok; ++q) {
+            if (!mine_q(q)) {
+                if (in_diag++ == diag) { ++diag; in_diag = 0; }
+                continue;
+            }
+            if (DUO && diag >= 4 && !others_in) {
+                // from here on the order of additions matters
+                if (!(ok = wait_duo(duo_done, flags))) break;
+                others_in = true;
+            }
             const bool exact = diag_exact(K, diag);
             // rounding applies when the group goes on past its first product
             const bool rounds = !exact && group > 1 && diag > 0;
@@ -509,7 +576,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             };
             int coded = rounds && in_group == 0 && in_diag != diag ? 0 : Cfg::COLS;
             for (int c = 0; c < nch; ++c) {
-                const int t = q * nch + c, b = t % Cfg::NBUF;
+                const int t = t0 + c, b = t % Cfg::NBUF;
                 ok = mbar_wait(tfull0 + 8u * b, (uint32_t)((t / Cfg::NBUF) & 1), flags);
                 __syncwarp();
                 if (!ok) break;
@@ -635,12 +702,17 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (coded < Cfg::COLS && c >= 2) { code_columns(coded); coded += HC; }
             }
             if (!ok) break;
+            t0 += nch;
             // The sums are integer multiples of the smallest unit of this thread's
             // elements, 2^-24 bound; when that unit is a normal FP32 number so is
             // every nonzero sum, and the short widening is exact.
             const bool normal_sums = bound >= 0x1p-102f;
             ++in_group;
             const bool last = in_diag == diag || in_group == group;      // last product of its group
+            if (DUO && last && !first_in) {                              // product 0 is in the accumulator
+                if (!(ok = wait_duo(duo_first, flags))) break;
+                first_in = true;
+            }
             if (last) {
                 // C <- fl64(C + (hi + lo)) in L2, column by column (product 0: a plain store).
                 // The common cases (no low words, normal unit) are branches of their own
@@ -685,6 +757,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     }
                 }
                 in_group = 0;
+                if (DUO && duo && q == 0) signal_duo(duo_first, rank);
             } else if (rounds) {
                 // Round the running sums as the addition of this product to the result
                 // rounds it.  (lock holds: the unit is normal.)
@@ -759,8 +832,14 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // one of its rows is live (a pair's second CTA may reach past the last
         // row).  Lanes of rows past M read their accumulator elements (inside the
         // tile, never written) and the copies leave those rows out.
+        if (DUO && duo && __all_sync(0xFFFFFFFFu, ok)) {
+            signal_duo(duo_done, rank);
+            if (!others_in) ok = wait_duo(duo_done, flags);
+        }
+        // the half of the tile's columns that this CTA of a duo writes
+        const bool writes = !DUO || (duo ? (uint32_t)(cq >> 1) == rank : rank == 0);
         const bool warp_ok = __all_sync(0xFFFFFFFFu, ok), warp_live = __any_sync(0xFFFFFFFFu, live);
-        if (warp_ok && warp_live && c_tma && !TAIL) {
+        if (warp_ok && warp_live && writes && c_tma && !TAIL) {
             // the accumulator holds every product now (this thread's own reductions,
             // same addresses, so they precede these loads): C <- acc through the TMA
             // engine.  Each 32 x 16 piece of the warp's rows (4 KB, two alternating
@@ -802,7 +881,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
             if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
-        } else if (ok && live && !(c_tma && !TAIL)) {
+        } else if (ok && live && writes && !(c_tma && !TAIL)) {
             // the accumulator holds every product now (this thread's own reductions,
             // same addresses, so they precede these loads): C <- acc (+ the merged tail)
             const float *trow = TAIL ? T + (int64_t)(row < M ? row : 0) * ldt + n0 + cq * Cfg::COLS : nullptr;
@@ -831,7 +910,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
     tc_fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync();               // the leader's MMAs are done with both CTAs
+    if constexpr (PAIR || DUO) cluster_sync();        // the leader's MMAs, a duo's signals are done with both CTAs
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
@@ -844,7 +923,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 // waves when narrower tiles take the rest), one CTA each, or with PAIR one
 // cluster of two CTAs each; or with wide_first >= 0 (pairs, BN = 128) `tiles`
 // 256 x 128 halves of the 256 x 256 tiles from raster index wide_first on.
-template <int BN, bool ROWCOL, bool TAIL, bool PAIR>
+template <int BN, bool ROWCOL, bool TAIL, bool PAIR, bool DUO>
 cudaError_t run_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp, int64_t ldcomp,
                      const int32_t *vA, const int32_t *vB, int nprod, double *C, int64_t ldc, double *acc,
                      uint32_t *flags, cudaStream_t st, int64_t a_plane, const float *T, int64_t ldt, int64_t tiles,
@@ -857,11 +936,11 @@ cudaError_t run_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const 
         return cudaErrorInvalidValue;
     CUtensorMap tc = {};
     const int c_tma = make_c_map_f64(&tc, C, M, N, ldc) ? 1 : 0;
-    auto kern = prodsum_f64w_kernel<BN, ROWCOL, TAIL, PAIR>;
+    auto kern = prodsum_f64w_kernel<BN, ROWCOL, TAIL, PAIR, DUO>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((PAIR ? 2 : 1) * tiles));
+    cfg.gridDim = dim3((unsigned)((PAIR || DUO ? 2 : 1) * tiles));
     cfg.blockDim = dim3(Cfg::THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = st;
@@ -873,7 +952,7 @@ cudaError_t run_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const 
     at[1].val.clusterDim.y = 1;
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = PAIR ? 2 : 1;
+    cfg.numAttrs = PAIR || DUO ? 2 : 1;
     e = cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, c_tma, (int)M, (int)N, (int)K, nprod, vA, vB, C, ldc, acc, flags, T,
                            ldt, wide_first);
     if (e != cudaSuccess) return e;
@@ -884,17 +963,22 @@ template <int BN, bool PAIR>
 cudaError_t dispatch_f64w(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const uint16_t *Bp, int64_t ldcomp,
                           const int32_t *vA, const int32_t *vB, int nprod, double *C, int64_t ldc, double *acc,
                           uint32_t *flags, cudaStream_t st, int64_t a_plane, bool rowcol, const float *T, int64_t ldt,
-                          int64_t tiles, int wide_first)
+                          int64_t tiles, int wide_first, bool duo = false)
 {
     if (T) {                                          // merged tail: whole-matrix levels only
         if (rowcol) return cudaErrorInvalidValue;
-        return run_f64w<BN, false, true, PAIR>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
+        return run_f64w<BN, false, true, PAIR, false>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
                                                T, ldt, tiles, wide_first);
     }
     if (rowcol)
-        return run_f64w<BN, true, false, PAIR>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
+        return run_f64w<BN, true, false, PAIR, false>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane,
                                                T, ldt, tiles, wide_first);
-    return run_f64w<BN, false, false, PAIR>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane, T,
+    if constexpr (BN < 256 && !PAIR) {
+        if (duo)
+            return run_f64w<BN, false, false, false, true>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st,
+                                                           a_plane, T, ldt, tiles, wide_first);
+    }
+    return run_f64w<BN, false, false, PAIR, false>(M, N, K, Ap, Bp, ldcomp, vA, vB, nprod, C, ldc, acc, flags, st, a_plane, T,
                                             ldt, tiles, wide_first);
 }
 

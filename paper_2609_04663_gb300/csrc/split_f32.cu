@@ -239,10 +239,26 @@ struct F32Operand {
     bool transpose;
 };
 
+// Block i of an operand's share (the orientation is a template parameter so that
+// a launch of small operands, which lasts about as long as its instructions take
+// to arrive, holds no more code than it runs).
+template <bool TRANSPOSE>
+__device__ __forceinline__ uint32_t split_operand(const F32Operand &o, int64_t ldcomp, WsHeader *ws, int64_t i,
+                                                  uint32_t (&sm)[3][kTile][kTile / 2])
+{
+    if constexpr (TRANSPOSE)
+        return split_f32_transpose_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i, o.n, sm);
+    else
+        return o.ax > 0 ? split_f32_rows_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i % o.ax, i / o.ax,
+                                              o.n / o.ax)
+                        : split_f32_rowtile_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, i, o.n);
+}
+
 // Both operands of an FP32 GEMM in one launch: blocks [0, a.n) split A, the next
 // b.n split B, and the last nC set the M x N result C to zero (a product-sum
 // that adds its K-parts into C needs it cleared).
-__global__ void __launch_bounds__(kThreads)
+template <bool TA, bool TB>
+__global__ void __launch_bounds__(kThreads, 4)
 split_f32_gemm_kernel(const __grid_constant__ F32Operand oa, const __grid_constant__ F32Operand ob, int64_t ldcomp,
                       WsHeader *ws, float *__restrict__ C, int64_t M, int64_t N, int64_t ldc, int64_t nC)
 {
@@ -254,13 +270,9 @@ split_f32_gemm_kernel(const __grid_constant__ F32Operand oa, const __grid_consta
     const int64_t nA = oa.n, nB = ob.n;
     const int64_t b = blockIdx.x;
     if (b < nA + nB) {
-        const F32Operand &o = b < nA ? oa : ob;
-        const int64_t i = b < nA ? b : b - nA;
-        const uint32_t amax =
-            o.transpose ? split_f32_transpose_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i, o.n, sm)
-            : o.ax > 0 ? split_f32_rows_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, ws, i % o.ax, i / o.ax,
-                                             o.n / o.ax)
-                       : split_f32_rowtile_body(o.X, o.rows, o.cols, o.ldx, o.comps, ldcomp, o.plane, i, o.n);
+        uint32_t amax;
+        if (b < nA) amax = split_operand<TA>(oa, ldcomp, ws, b, sm);
+        else amax = split_operand<TB>(ob, ldcomp, ws, b - nA, sm);
         // the flag word is cleared by the operation before this launch, which
         // may still be running when this kernel is its programmatic dependent
         griddep_wait();
@@ -344,7 +356,9 @@ cudaError_t launch_split_f32_gemm(const float *A, int64_t M, int64_t K, int64_t 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, split_f32_gemm_kernel, a, b, ldcomp, ws, C, M, N, ldc, nC);
+    auto kern = ta ? (tb ? split_f32_gemm_kernel<true, true> : split_f32_gemm_kernel<true, false>)
+                   : (tb ? split_f32_gemm_kernel<false, true> : split_f32_gemm_kernel<false, false>);
+    e = cudaLaunchKernelEx(&cfg, kern, a, b, ldcomp, ws, C, M, N, ldc, nC);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -53,7 +53,19 @@ rc_max_pass(const double *__restrict__ X, int64_t rows, int64_t cols, int64_t ld
             if (ff && ff[i] >= L) continue;
             for (int l = 0; l < L; ++l) v[l] = vrc[l * nvec + i];
             unsigned long long m = 0;
-            for (int64_t j = lane_id(); j < cols; j += 32) take(X[i * ldx + j], v, m);
+            const double *row = X + i * ldx;
+            int64_t j = lane_id();
+            // level 0 is bound by memory latency: eight loads of a lane in flight
+            if (L == 0) {
+                for (; j + 7 * 32 < cols; j += 8 * 32) {
+                    double x[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) x[k] = row[j + 32 * k];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) take(x[k], v, m);
+                }
+            }
+            for (; j < cols; j += 32) take(row[j], v, m);
             m = warp_max(m);
             if (lane_id() == 0) maxbits[i] = m;
         }
@@ -67,7 +79,17 @@ rc_max_pass(const double *__restrict__ X, int64_t rows, int64_t cols, int64_t ld
             if (j < cols && !(ff && ff[j] >= L)) {
                 for (int l = 0; l < L; ++l) v[l] = vrc[l * nvec + j];
                 unsigned long long m = 0;
-                for (int64_t i = i0; i < i1; ++i) take(X[i * ldx + j], v, m);
+                int64_t i = i0;
+                if (L == 0) {
+                    for (; i + 7 < i1; i += 8) {
+                        double x[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) x[k] = X[(i + k) * ldx + j];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) take(x[k], v, m);
+                    }
+                }
+                for (; i < i1; ++i) take(X[i * ldx + j], v, m);
                 if (m) atomicMax(&maxbits[j], m);
             }
         }
