@@ -129,9 +129,8 @@ cudaError_t launch_prodsum_f64_narrow(int64_t M, int64_t N, int64_t K, const uin
                                      bool rowcol, const float *T, int64_t ldt, int cols, bool pair, int64_t tiles,
                                       int wide_first, bool duo);
 
-// Bytes of the FP64 product-sum's accumulator, enough for either tile shape:
-// one FP64 tile of 128 x 128 (narrow kernel) or 128 x 256 (wide kernel) per
-// CTA tile.
+// Bytes of the FP64 product-sum's accumulator: 128-row stripes of roundup(N, 256)
+// columns, whatever tile shape runs.
 inline size_t f64_acc_bytes(int64_t M, int64_t N)
 {
     const size_t tm = (size_t)((M + 127) / 128);
