@@ -227,7 +227,12 @@ __device__ __forceinline__ bool wait_duo(uint32_t bar, uint32_t *flags)
 constexpr uint32_t kCodeKeep = 0, kCodeEach = 1;
 __device__ __forceinline__ uint32_t code_byte(uint32_t word, int k) { return (word >> (8 * k)) & 0xFFu; }
 // Exponent fields of the four rounding constants of a code word: its bytes
-// plus the field of 2^-25 u (at most 254 in all).
+// plus the field of 2^-25 u, bound_bits >> 23 minus 49.  No byte may borrow from or
+// carry into the next, or be 255.  With lock, e0 + 8 - 8 (d - 1) >= -76 and e0 <= 100
+// give 51 <= bound_bits >> 23 <= 227 on the diagonals that round (1 .. d - 1), and the
+// largest byte is 227 - 49 + 48 + kMaxRoundBits = 246; the all-zero columns' word
+// (level exponent 60, whatever the row) stays between 51 and 247 and its bytes are
+// kCodeKeep, the all-zero rows take the level of another row.
 __device__ __forceinline__ uint32_t round_fields(uint32_t word, uint32_t bound_bits)
 {
     return (word & 0x7F7F7F7Fu) + ((bound_bits >> 23) - 49u) * 0x01010101u;
@@ -486,6 +491,10 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             lock = lsum->lock != 0 && lsum->max_a <= 60 && lsum->max_b <= 60 && lsum->max_a + lsum->max_b <= 100 &&
                    lsum->max_a >= lsum->min_a && lsum->max_b >= lsum->min_b &&
                    lsum->min_a + lsum->min_b + 8 - 8 * (d - 1) >= -76;
+            // An all-zero row has no level: take one of the range that lock has checked, so
+            // that the row's bounds and rounding constants are normal numbers for every column
+            // (with level 0 a constant's exponent could be all ones, and 0 + inf - inf a NaN).
+            if (lock && v0 == kZeroLevel) row_e = lsum->min_a;
             lvl_min = 0x7FFFFFFF;
 #pragma unroll 4
             for (int j = 0; j < Cfg::COLS; ++j) lvl_min = min(lvl_min, lvl[j]);
