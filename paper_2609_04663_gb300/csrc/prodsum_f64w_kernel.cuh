@@ -208,9 +208,30 @@ __device__ __forceinline__ void signal_duo(uint32_t bar, uint32_t rank)
                      : "memory");
     __syncwarp();
 }
+// Bounded wait for phase 0 of a duo's barrier: mbar_wait's polling with an
+// acquire at cluster scope, since the writes it orders are the other CTA's (a
+// wait that acquires at CTA scope does not synchronise with that CTA's release).
 __device__ __forceinline__ bool wait_duo(uint32_t bar, uint32_t *flags)
 {
-    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, 0, flags));
+    auto poll = [bar] {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar)
+            : "memory");
+        return ok != 0;
+    };
+    bool ok = poll();
+    const unsigned long long t0 = ok ? 0 : globaltimer_ns();
+    for (uint32_t it = 1; !ok && it < (1u << 30); ++it) {
+        ok = poll();
+        if (!ok && (it & 63u) == 0u && globaltimer_ns() - t0 > kWaitLimitNs) break;
+    }
+    if (!ok) atomicOr(flags, (uint32_t)EMU_FLAG_TIMEOUT);
+    ok = __all_sync(0xFFFFFFFFu, ok);
     __threadfence();
     return ok;
 }
