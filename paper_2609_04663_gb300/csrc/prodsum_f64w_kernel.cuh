@@ -472,6 +472,9 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // a pair's second CTA may lie wholly below the last row, past the
         // accumulator's stripes: its threads touch neither the accumulator nor C
         const bool live = !PAIR || row < M;
+        // where code_columns reads the accumulator: rows past M read the first stripe (any
+        // address of it will do, the value is dropped)
+        const double *hacc = live ? tacc : acc;
         // the low words live in one half of this thread's C words until their group is reduced
         float *lrow = reinterpret_cast<float *>(crow) + (DUO ? rank : 0u);
         uint32_t *codes = reinterpret_cast<uint32_t *>(base_ptr + Cfg::CODE_OFF) + dt;   // word w at w * DRAIN_THREADS
@@ -576,12 +579,17 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // from the accumulator H (every earlier product is in it; this thread's own
             // reductions, so they precede the loads).  HC columns per chunk, from the third
             // chunk on, in time the warp would wait for partials, and the rest after the
-            // last chunk.
+            // last chunk.  No branches in it: with a branch per element (a load for live rows only,
+            // the cases of the code) the loads were not in flight together and 128 columns took
+            // 64,000 clocks, now 20,000 (21 products of 16384 x 256 x 256: 298 -> 259 us, of
+            // 3000 x 3000 x 300: 440 -> 358).
             constexpr int HC = BN == 256 ? 16 : 8;
             auto code_columns = [&](int j0) {
                 double hd[HC];
 #pragma unroll
-                for (int k = 0; k < HC; ++k) hd[k] = live ? ld_cg_f64(tacc + (j0 + k) * kBM) : 0.0;
+                for (int k = 0; k < HC; ++k) hd[k] = ld_cg_f64(hacc + (j0 + k) * kBM);
+#pragma unroll
+                for (int k = 0; k < HC; ++k) hd[k] = live ? hd[k] : 0.0;
 #pragma unroll
                 for (int w = 0; w < HC / 4; ++w) {
                     uint32_t cw = 0;
@@ -592,13 +600,10 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         // g = 2^n u: exponent fields e - 1023 - 52 - (field of 2^24 u - 127 - 24)
                         const int n = (int)(xh >> 20) - 924 - (int)(bits_of(j0 + 4 * w + k) >> 23);
                         const uint32_t mh = xh & 0xFFFFFu;
-                        uint32_t code = kCodeKeep;
-                        if ((n >= 0 && mh == 0xFFFFFu) || (n > 0 && mh == 0u) || n > kMaxRoundBits) {
-                            code = kCodeEach;
-                            each = true;
-                        } else if (n > 0) {
-                            code = (uint32_t)(n + 48) | (((uint32_t)__double2loint(h) & 1u) << 7);
-                        }
+                        const bool edge = ((n >= 0) & (mh == 0xFFFFFu)) | ((n > 0) & (mh == 0u)) | (n > kMaxRoundBits);
+                        const uint32_t odd = ((uint32_t)__double2loint(h) & 1u) << 7;
+                        each |= edge;
+                        const uint32_t code = edge ? kCodeEach : n > 0 ? (uint32_t)(n + 48) | odd : kCodeKeep;
                         cw |= code << (8 * k);
                     }
                     codes[(j0 / 4 + w) * Cfg::DRAIN_THREADS] = cw;
