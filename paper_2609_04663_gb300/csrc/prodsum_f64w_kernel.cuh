@@ -79,8 +79,13 @@ struct F64WCfgT {
     static constexpr int BN = BN_, KB = 64, NBUF = BN == 256 ? 2 : 4;
     static constexpr int BH = PAIR ? BN / 2 : BN;                       // B rows staged by this CTA
     static constexpr int A_TILE = kBM * KB * 2, B_TILE = BH * KB * 2;   // 16 KB + 8 to 32 KB
-    static constexpr int STAGE = A_TILE + B_TILE;
-    static constexpr int STAGES = 196608 / STAGE;                        // 4 x 48, 6 x 32 or 8 x 24 KB
+    // K-blocks of 64 per stage.  The 128 x 128 tiles run where few CTAs are at work and
+    // wait for operands: with two blocks (adjacent 128-byte pieces of every plane
+    // row requested together) 1024 x 1024 x 32768 / 21 takes 3090 us, with one 3620.
+    static constexpr int SUB = BN == 128 && !PAIR ? 2 : 1, KSPAN = KB * SUB;
+    static constexpr int STAGE = SUB * (A_TILE + B_TILE);
+    static constexpr int STAGES = 196608 / STAGE;                        // 4 x 48, 3 x 64, 6 x 32 or 8 x 24 KB
+    static constexpr int B_OFF = SUB * A_TILE;                           // A blocks, then B blocks
     static constexpr uint32_t SWZ = 2u, SBO = 1024u;                     // 128-byte swizzle
     // warpgroup 0: TMA producer (warp 0), MMA issuer + TMEM owner (warp 1), two
     // idle warps; then the drain warps: sixteen of BN / 4 columns each, or with
@@ -104,7 +109,7 @@ struct F64WCfgT {
     static constexpr int REG_CTRL = BN == 256 ? 40 : 32, REG_DRAIN = BN == 256 ? 232 : 112,
                          REG_LAUNCH = BN == 256 ? 168 : 96;
     static_assert(NBUF * BN <= 512, "TMEM budget");
-    static_assert(kKChunk % KB == 0, "a K-chunk is a whole number of stages");
+    static_assert(kKChunk % KSPAN == 0, "a K-chunk is a whole number of stages");
     static_assert(8 * NBARS + 8 + 20 <= 256, "barrier area");
     static_assert(SMEM <= 232448, "shared memory per CTA");
     static_assert(128 * REG_CTRL + DRAIN_THREADS * REG_DRAIN <= THREADS * REG_LAUNCH,
@@ -368,7 +373,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp < Cfg::FIRST_DRAIN) {
       regs_dec<Cfg::REG_CTRL>();
       if (warp == 0 && lane == 0) {
-        // ---------------- TMA producer: for product, for chunk, for 64-wide K-block of the chunk
+        // ---------------- TMA producer: for product, for chunk, for stage (KSPAN of K) of the chunk
         int L = 0, s = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -376,21 +381,24 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             if (!mine_q(q)) continue;
             const int ia = kDiag[q][0], jb = kDiag[q][1];
             for (int c = 0; c < nch && ok; ++c) {
-                const int kbs = min(kKChunk / Cfg::KB, (K - c * kKChunk + Cfg::KB - 1) / Cfg::KB);
+                const int kbs = min(kKChunk / Cfg::KSPAN, (K - c * kKChunk + Cfg::KSPAN - 1) / Cfg::KSPAN);
                 for (int u = 0; u < kbs; ++u, ++L) {
                     if (!(ok = mbar_wait(empty0 + 8u * s, ph ^ 1u, flags))) break;
                     const uint32_t st = base + (uint32_t)(s * Cfg::STAGE), fb = full0 + 8u * s;
-                    const int k0 = c * kKChunk + u * Cfg::KB;
+                    const int k0 = c * kKChunk + u * Cfg::KSPAN;
                     if constexpr (PAIR) {
                         // both CTAs' copies are counted on the leader's full barrier
                         const uint32_t fl = peer_addr(fb, 0);
                         if (rank == 0) mbar_arrive_expect_tx(fb, 2 * Cfg::STAGE);
                         tma_load_3d_pair(st, &tmA, fl, k0, m0, ia);
-                        tma_load_3d_pair(st + Cfg::A_TILE, &tmB, fl, k0, n0 + (int)rank * Cfg::BH, jb);
+                        tma_load_3d_pair(st + Cfg::B_OFF, &tmB, fl, k0, n0 + (int)rank * Cfg::BH, jb);
                     } else {
-                        mbar_arrive_expect_tx(fb, Cfg::STAGE);
-                        tma_load_3d(st, &tmA, fb, k0, m0, ia);
-                        tma_load_3d(st + Cfg::A_TILE, &tmB, fb, k0, n0, jb);
+                        const int blocks = Cfg::SUB == 1 || k0 + Cfg::KB < K ? Cfg::SUB : 1;   // a block wholly past K is left out
+                        mbar_arrive_expect_tx(fb, (uint32_t)(blocks * (Cfg::A_TILE + Cfg::B_TILE)));
+                        for (int h = 0; h < blocks; ++h) {
+                            tma_load_3d(st + h * Cfg::A_TILE, &tmA, fb, k0 + h * Cfg::KB, m0, ia);
+                            tma_load_3d(st + Cfg::B_OFF + h * Cfg::B_TILE, &tmB, fb, k0 + h * Cfg::KB, n0, jb);
+                        }
                     }
                     if (++s == Cfg::STAGES) { s = 0; ph ^= 1u; }
                 }
@@ -412,15 +420,16 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         // issues: control flow and operands are then uniform, and the descriptors
         // need no move from vector to uniform registers before every MMA.
         constexpr uint32_t idesc = make_idesc_bf16(PAIR ? 2 * kBM : kBM, BN);
-        // descriptors of stage 0; stage s and 16-wide K step kk add (s STAGE + 32 kk) / 16
-        const uint64_t ad0 = make_sdesc(base, Cfg::SBO, Cfg::SWZ), bd0 = make_sdesc(base + Cfg::A_TILE, Cfg::SBO, Cfg::SWZ);
+        // descriptors of stage 0; stage s, block h and 16-wide K step kk of it add their byte
+        // offsets / 16
+        const uint64_t ad0 = make_sdesc(base, Cfg::SBO, Cfg::SWZ), bd0 = make_sdesc(base + Cfg::B_OFF, Cfg::SBO, Cfg::SWZ);
         int s = 0, b = 0, c = 0;
         uint32_t ph = 0, tph = 0;
         bool ok = true;
         int nmine = 0;                                // products of this CTA
         for (int q = 0; q < nprod; ++q) nmine += mine_q(q) ? 1 : 0;
         for (int t = 0; t < nmine * nch && ok; ++t) {
-            const int kbs = min(kKChunk / Cfg::KB, (K - c * kKChunk + Cfg::KB - 1) / Cfg::KB);
+            const int kbs = min(kKChunk / Cfg::KSPAN, (K - c * kKChunk + Cfg::KSPAN - 1) / Cfg::KSPAN);
             if (!(ok = __all_sync(0xFFFFFFFFu, mbar_wait(tempty0 + 8u * b, tph ^ 1u, flags)))) break;
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(b * BN);
@@ -429,11 +438,16 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 tc_fence_after();
                 const uint32_t off = (uint32_t)(s * (Cfg::STAGE / 16));
                 const uint64_t ad = ad0 + off, bd = bd0 + off;
+                const bool second = Cfg::SUB == 1 || c * kKChunk + u * Cfg::KSPAN + Cfg::KB < K;
                 if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < Cfg::KB / 16; ++kk) {
-                        if constexpr (PAIR) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (u | kk) != 0);
-                        else mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (u | kk) != 0);
+                    for (int kk = 0; kk < Cfg::KSPAN / 16; ++kk) {
+                        // K step kk lies 32 bytes a step into its 64-wide block
+                        const int h = kk / (Cfg::KB / 16), o = 2 * (kk % (Cfg::KB / 16));
+                        if (h > 0 && !second) break;
+                        const uint64_t a = ad + h * (Cfg::A_TILE / 16) + o, w = bd + h * (Cfg::B_TILE / 16) + o;
+                        if constexpr (PAIR) mma_bf16_pair(d, a, w, idesc, (u | kk) != 0);
+                        else mma_bf16(d, a, w, idesc, (u | kk) != 0);
                     }
                     if constexpr (PAIR) mma_commit_pair(empty0 + 8u * s);
                     else mma_commit(empty0 + 8u * s);
