@@ -20,9 +20,10 @@
 //
 // Eight or sixteen drain warps (two or four per TMEM lane quarter) sum
 // partials exactly in FP32 registers: plain additions while the running sum
-// stays below 2^24 u; past that either a carry of the coarse part (multiples
-// of 2^12 u) into a low word kept in C, or TwoSums whose errors are summed
-// into that low word.
+// stays below 2^24 u; past that the sum goes into the FP64 accumulator where
+// that is exact (below), else a carry of the coarse part (multiples of 2^12 u)
+// into a low word kept in C, or TwoSums whose errors are summed into that low
+// word.
 //
 // Algorithm 2 adds every product once into the FP64 result, C <- fl64(C +
 // A_i B_j), in diagonal order.  The accumulator is an FP64 buffer in the
@@ -546,7 +547,9 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         };
 
         float hi[Cfg::COLS];
-        uint32_t dirty = 0;                                   // 16-column groups whose low part lives in C
+        uint32_t dirty = 0;                                   // 16-column groups whose low part lives in C; from bit
+                                                              // 16 on, those whose sums of product 0 have begun
+                                                              // to be in the accumulator
         bool each = false;                                    // some element is reduced after every product
         int diag = 0, in_diag = 0, in_group = 0;              // product q: diagonal, place in it and in its group
         bool ok = true;
@@ -581,13 +584,15 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // while a group's sums are rounded they stay below (1 - 2^-4) 2^24 u (kMaxRoundBits)
             const float limit = rounds ? 0.9375f * bound : bound;
             const int abits_lim = rounds ? abits - 0x100000 : abits;
-            // Carry instead of TwoSums when all elements share the unit u = 2^-24 bound
-            // (levels per matrix) and the split constant 1.5 * 2^35 u is finite.  A
+            // What happens to sums that would reach 2^24 u.
+            // 2: they are reduced into the accumulator, while every addition to it is exact.
+            // 1: a carry instead of TwoSums (0), when all elements share the unit u = 2^-24
+            // bound (levels per matrix) and the split constant 1.5 * 2^35 u is finite.  A
             // carry splits the running sum and the partial (each at most 2^24 u) at
             // multiples of 2^12 u and moves both coarse parts (together at most
             // 2^25 u) to the low word in C, which stays exact below 2^36 u, i.e. for
             // up to 2^11 carries.
-            const bool carry = !ROWCOL && bound > 0.0f && bound <= 0x1p116f && nch <= 2048;
+            const int past = exact && lock && first_in ? 2 : !ROWCOL && bound > 0.0f && bound <= 0x1p116f && nch <= 2048 ? 1 : 0;
             const int a_row = (ROWCOL && row < M) ? vA[(int64_t)kDiag[q][0] * M + row] : kZeroLevel;
             // The first product of a group whose sums are rounded: g of elements j0 .. j0 + HC - 1
             // from the accumulator H (every earlier product is in it; this thread's own
@@ -685,9 +690,30 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         for (int j = 0; j < 16; ++j) hi[h + j] = __uint_as_float(ps[g + j]);
                         continue;
                     }
+                    if (past == 2) {
+                        // some sum would reach 2^24 u, and every addition to the accumulator is
+                        // exact up to this diagonal: reduce the sums now and go on from the
+                        // partials (read again from TMEM).  Non-negative operands come here every
+                        // few chunks of product 0; the accumulator's columns are 256 contiguous
+                        // bytes of a warp, where the low words below are 32 sectors each way
+                        // (4096 x 4096 x 2048 / 6, entries in [1/2, 1]: 2058 -> 580 us).
+                        const bool store = q == 0 && !((dirty >> (16 + h / 16)) & 1u);
+#pragma unroll
+                        for (int j = h; j < h + 16; ++j) {
+                            const double x = widen_normal(hi[j]);
+                            if (live && store) tacc[j * kBM] = x;
+                            if (live && !store) red_add_f64(tacc + j * kBM, x);
+                        }
+                        if (q == 0) dirty |= 0x10000u << (h / 16);
+                        tmem_ld16(tcol + (uint32_t)(b * BN + h), p16);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int jj = 0; jj < 16; ++jj) hi[h + jj] = __uint_as_float(p16[jj]);
+                        continue;
+                    }
                     tmem_ld16(tcol + (uint32_t)(b * BN + h), p16);
                     tmem_ld_wait();
-                    if (carry) {
+                    if (past == 1) {
                         // rare: some sum would reach 2^24 u.  Split the running sum and
                         // the partial (read again from TMEM) at multiples of 2^12 u by the add-subtract
                         // projection; the coarse parts go to the low word in C, the
@@ -785,7 +811,7 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     const bool low = (dirty >> (h / 16)) & 1u;
                     if (!__any_sync(0xFFFFFFFFu, low) && normal_sums) {
                         if (!live) continue;
-                        if (q == 0) {
+                        if (q == 0 && !((dirty >> (16 + h / 16)) & 1u)) {
 #pragma unroll
                             for (int j = h; j < h + 16; ++j) tacc[j * kBM] = widen_normal(hi[j]);
                         } else {
