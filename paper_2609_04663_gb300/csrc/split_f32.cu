@@ -338,8 +338,10 @@ cudaError_t launch_split_f32_gemm(const float *A, int64_t M, int64_t K, int64_t 
         } else if (o->transpose) {
             o->n = grid_for(tiles(*o), 152 * 4);
         } else {
+            // at most 608 (or one row of blocks): of 620, which rows of 40,000 would round up
+            // to, the last 12 ran alone for as long as all the others
             o->ax = (o->cols + 8 * kThreads - 1) / (8 * kThreads);
-            const int64_t want = (152 * 4 + o->ax - 1) / o->ax;
+            const int64_t want = o->ax < 152 * 4 ? 152 * 4 / o->ax : 1;
             o->n = o->ax * (o->rows < want ? o->rows : want);
         }
     }
