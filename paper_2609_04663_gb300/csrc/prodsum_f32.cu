@@ -68,15 +68,33 @@ __device__ __forceinline__ void reduce_tile(uint32_t tmem, int quarter, int c0, 
 // red.global.add.v4 in store_tile / reduce_tile touches 32 cache lines, one
 // per row, and those epilogues took 4.7 us per 128 x 256 tile and 2.0 us per
 // 128 x 128 tile on GB300.
+// The general GEMM's scaling (ab = 1: C <- fl(alpha P), ab = 2: C <- fl(fl(alpha P) +
+// fl(beta C)), each operation rounded once) is applied on the way; the pieces of C
+// it reads are all requested at once, by bulk tensor loads into the buffers
+// they leave from, counted on the warp's barrier `cbar` (8192 x 8192 x 64, beta = 1/2:
+// 160 us; with epilogue_rows' loads and stores of single words 304, with the
+// product stored and a separate pass 290).
 template <bool REDUCE>
 __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int ncols, int m0, int n0, int M, int N,
-                                             const CUtensorMap *cmap, uint32_t stage)
+                                             const CUtensorMap *cmap, uint32_t stage, float alpha, float beta, int ab,
+                                             uint32_t cbar, uint32_t *flags)
 {
     tc_fence_after();
     const uint32_t lane = lane_id();
     const uint32_t slots = stage + (uint32_t)(quarter * ncols) * 128u;     // 32 rows x 4 bytes per column
     // pieces wholly past the last row or column are neither staged nor copied
     const int cols = m0 + quarter * 32 < M ? min(ncols, N - n0) : 0;
+    if (!REDUCE && ab == 2 && cols > 0) {
+        if (lane == 0) {
+            mbar_arrive_expect_tx(cbar, (uint32_t)((cols + 31) / 32) * 4096u);
+            for (int c = 0; c < cols; c += 32)
+                tma_load_2d(slots + (uint32_t)c * 128u, cmap, cbar, n0 + c, m0 + quarter * 32);
+        }
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(cbar, 0, flags))) {
+            (void)mbar_wait(cbar, 0, flags, 100000000ull);        // copies in flight
+            return;
+        }
+    }
 #pragma unroll 1
     for (int c = 0; c < cols; c += 32) {
         uint32_t v[32];
@@ -84,6 +102,21 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
         tmem_ld_wait();
         // row `lane` of the piece: 16-byte chunk j at chunk j ^ (lane % 8), conflict-free
         const uint32_t buf = slots + (uint32_t)c * 128u, row = buf + lane * 128u;
+        if (!REDUCE && ab != 0) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__fmul_rn(alpha, __uint_as_float(v[j])));
+            if (ab == 2) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    uint32_t old[4];
+                    ld_shared_v4(row + ((uint32_t)(j ^ (int)(lane & 7u)) << 4), old[0], old[1], old[2], old[3]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        v[4 * j + k] = __float_as_uint(__fadd_rn(__uint_as_float(v[4 * j + k]),
+                                                                 __fmul_rn(beta, __uint_as_float(old[k]))));
+                }
+            }
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j)
             st_shared_v4(row + ((uint32_t)(j ^ (int)(lane & 7u)) << 4), v[4 * j], v[4 * j + 1], v[4 * j + 2],
@@ -104,14 +137,13 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
     __syncwarp();
 }
 
-// Epilogue of one warp for a C that no tensor map describes, or with the
-// general GEMM's scaling (ab = 1: C <- fl(alpha P), ab = 2: C <- fl(fl(alpha P) +
-// fl(beta C)), each operation rounded once): each 32 x 32 piece is turned in
+// Epilogue of one warp for a C that no tensor map describes, with the general
+// GEMM's scaling as in epilogue_tma: each 32 x 32 piece is turned in
 // shared memory (stage memory, free once every MMA has completed; rows of 33
 // words, conflict-free both ways) so that a warp reads and writes whole row
-// segments, the rows of C it scales requested before the piece is read from
-// TMEM.  One lane per row, as in store_tile, touches a cache line per lane: at
-// 1537 x 2050 x 1100 that and a separate alpha / beta pass took 28 of 90 us.
+// segments, the rows of C it scales requested a piece ahead.  One lane per row,
+// as in store_tile, touches a cache line per lane: at 1537 x 2050 x 1100 that
+// and a separate alpha / beta pass took 28 of 90 us.
 __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int ncols, int m0, int n0, int M, int N,
                                               float *__restrict__ C, int64_t ldc, float alpha, float beta, int ab,
                                               uint8_t *stage)
@@ -120,14 +152,21 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int nc
     const int lane = (int)lane_id(), row0 = m0 + quarter * 32, nr = min(32, M - row0);
     float *buf = reinterpret_cast<float *>(stage) + quarter * (32 * 33);
     const int cols = nr > 0 ? min(ncols, N - n0) : 0;
+    float *cp = C + (int64_t)row0 * ldc + n0 + lane;
+    float next[32];                                  // C of the next piece (column c + lane, 32 rows)
+    auto load_c = [&](int c) {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) next[r] = (c + lane < cols && r < nr) ? cp[(int64_t)r * ldc + c] : 0.0f;
+    };
+    if (ab == 2) load_c(0);
 #pragma unroll 1
     for (int c = 0; c < cols; c += 32) {
         const bool mine = c + lane < cols;
-        float *cp = C + (int64_t)row0 * ldc + n0 + c + lane;
         float old[32];
         if (ab == 2) {
 #pragma unroll
-            for (int r = 0; r < 32; ++r) old[r] = (mine && r < nr) ? cp[(int64_t)r * ldc] : 0.0f;
+            for (int r = 0; r < 32; ++r) old[r] = next[r];
+            load_c(c + 32);
         }
         uint32_t v[32];
         tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
@@ -140,7 +179,7 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int nc
             float out = buf[r * 33 + lane];
             if (ab != 0) out = __fmul_rn(alpha, out);
             if (ab == 2) out = __fadd_rn(out, __fmul_rn(beta, old[r]));
-            if (mine && r < nr) cp[(int64_t)r * ldc] = out;
+            if (mine && r < nr) cp[(int64_t)r * ldc + c] = out;
         }
         __syncwarp();
     }
@@ -164,7 +203,7 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - raw);
     const uint32_t full0 = base + Cfg::BAR_OFF, empty0 = full0 + 8u * STAGES;
-    const uint32_t accum_bar = empty0 + 8u * STAGES;
+    const uint32_t accum_bar = empty0 + 8u * STAGES, cbar0 = full0 + Cfg::CBAR;   // cbar0: one per epilogue warp
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + Cfg::BAR_OFF + 16 * STAGES + 8);
 
     const int warp = threadIdx.x >> 5, lane = lane_id();
@@ -187,6 +226,7 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
         mbar_init(accum_bar, 1);
+        for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
         fence_mbar_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
@@ -223,10 +263,12 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // ---------------- epilogue: TMEM -> registers -> C (tcgen05.ld needs the
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
-        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
+        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
+                                                           cbar0 + 8u * (uint32_t)(warp & 3), flags);
         else if (ok && SPLIT == 1)
             epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
-        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
+        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
+                                                                   0, flags);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
     tc_fence_before();
@@ -261,7 +303,9 @@ struct F32PairCfg {
     static constexpr uint32_t SWZ = (KB == 64) ? 2u : 4u;
     static constexpr uint32_t SBO = 8u * KB * 2u;
     static constexpr int BAR_OFF = STAGES * STAGE;
+    static constexpr int CBAR = 128;                           // four barriers, after the pipeline's and the TMEM slot
     static constexpr int SMEM = BAR_OFF + 256 + 1024;
+    static_assert(16 * STAGES + 12 <= CBAR, "barrier area");
     static_assert(KB == 32 || KB == 64, "K-block must fill one 64 B or 128 B swizzle row");
     static_assert(BN % 32 == 0 && BN >= 64 && BN <= 256, "UMMA N of a pair");
     static_assert(SMEM <= 232448, "shared memory per CTA");
@@ -279,7 +323,7 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - raw);
     const uint32_t full0 = base + Cfg::BAR_OFF, empty0 = full0 + 8u * STAGES;
-    const uint32_t accum_bar = empty0 + 8u * STAGES;
+    const uint32_t accum_bar = empty0 + 8u * STAGES, cbar0 = full0 + Cfg::CBAR;   // cbar0: one per epilogue warp
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + Cfg::BAR_OFF + 16 * STAGES + 8);
     const int warp = threadIdx.x >> 5, lane = lane_id();
     const uint32_t rank = cluster_rank();
@@ -295,6 +339,7 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
         mbar_init(accum_bar, 1);
+        for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
         fence_mbar_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
@@ -354,10 +399,12 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // ---------------- epilogue of this CTA's 128 rows (tcgen05.ld needs the
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
-        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
+        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
+                                                           cbar0 + 8u * (uint32_t)(warp & 3), flags);
         else if (ok && SPLIT == 1)
             epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
-        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base);
+        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
+                                                                   0, flags);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
     tc_fence_before();
@@ -390,7 +437,7 @@ cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const u
     // the epilogue writes (or adds) C through a C tensor map when one exists
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
-    const int c_tma = ab == 0 && make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
+    const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
     auto kern = prodsum_f32_kernel<BN, KB, STAGES, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
@@ -426,7 +473,7 @@ cudaError_t run_f32_pair(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, co
         return cudaErrorInvalidValue;
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
-    const int c_tma = ab == 0 && make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
+    const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
     auto kern = prodsum_f32_pair_kernel<BN, KB, STAGES, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;

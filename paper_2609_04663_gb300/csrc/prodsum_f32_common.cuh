@@ -24,7 +24,9 @@ struct F32Cfg {
     static constexpr uint32_t SWZ = (KB == 64) ? 2u : 4u;       // 128-byte or 64-byte swizzle
     static constexpr uint32_t SBO = 8u * KB * 2u;               // bytes between 8-row groups
     static constexpr int BAR_OFF = STAGES * STAGE;
+    static constexpr int CBAR = 128;                            // four barriers, after the pipeline's and the TMEM slot
     static constexpr int SMEM = BAR_OFF + 256 + 1024;           // + barriers + alignment slack
+    static_assert(16 * STAGES + 12 <= CBAR, "barrier area");
     static constexpr int THREADS = 192;
     static_assert(KB == 32 || KB == 64, "K-block must fill one 64 B or 128 B swizzle row");
     static_assert(BN % 32 == 0 && BN >= 32 && BN <= 256, "UMMA N");
