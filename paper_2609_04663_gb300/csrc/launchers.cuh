@@ -133,10 +133,7 @@ cudaError_t launch_prodsum_f64_narrow(int64_t M, int64_t N, int64_t K, const uin
 // columns, whatever tile shape runs.
 inline size_t f64_acc_bytes(int64_t M, int64_t N)
 {
-    const size_t tm = (size_t)((M + 127) / 128);
-    const size_t narrow = tm * (size_t)((N + 127) / 128) * 128u * 128u * sizeof(double);
-    const size_t wide = tm * (size_t)((N + 255) / 256) * 128u * 256u * sizeof(double);
-    return narrow > wide ? narrow : wide;
+    return (size_t)((M + 127) / 128) * (size_t)((N + 255) / 256) * 128u * 256u * sizeof(double);
 }
 
 // General-GEMM epilogue: C <- fl(fl(alpha P) + fl(beta C)) (beta = 0: C <- fl(alpha P), C not read).

@@ -84,7 +84,7 @@ F64Plan f64_plan(int64_t M, int64_t N)
             p.tiles = tiles;
         }
     }
-    if (!forced && p.rows == 256) {
+    if (!forced && p.rows == 256 && p.cols == 256) {
         const int64_t slots = sms / 2, full = (p.tiles / slots) * slots, rem = p.tiles - full;
         const double t_mixed =
             (double)(full / slots) * 256.0 + (double)((2 * rem + slots - 1) / slots) * 128.0 / kRateHalf;
