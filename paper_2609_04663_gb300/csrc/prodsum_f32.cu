@@ -74,7 +74,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t tmem, int quarter, int c0, 
 // they leave from, counted on the warp's barrier `cbar` (8192 x 8192 x 64, beta = 1/2:
 // 160 us; with epilogue_rows' loads and stores of single words 304, with the
 // product stored and a separate pass 290).
-template <bool REDUCE>
+template <bool REDUCE, bool SCALE>
 __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int ncols, int m0, int n0, int M, int N,
                                              const CUtensorMap *cmap, uint32_t stage, float alpha, float beta, int ab,
                                              uint32_t cbar, uint32_t *flags)
@@ -84,7 +84,7 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
     const uint32_t slots = stage + (uint32_t)(quarter * ncols) * 128u;     // 32 rows x 4 bytes per column
     // pieces wholly past the last row or column are neither staged nor copied
     const int cols = m0 + quarter * 32 < M ? min(ncols, N - n0) : 0;
-    if (!REDUCE && ab == 2 && cols > 0) {
+    if (SCALE && ab == 2 && cols > 0) {
         if (lane == 0) {
             mbar_arrive_expect_tx(cbar, (uint32_t)((cols + 31) / 32) * 4096u);
             for (int c = 0; c < cols; c += 32)
@@ -102,7 +102,7 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
         tmem_ld_wait();
         // row `lane` of the piece: 16-byte chunk j at chunk j ^ (lane % 8), conflict-free
         const uint32_t buf = slots + (uint32_t)c * 128u, row = buf + lane * 128u;
-        if (!REDUCE && ab != 0) {
+        if (SCALE) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__fmul_rn(alpha, __uint_as_float(v[j])));
             if (ab == 2) {
@@ -144,6 +144,7 @@ __device__ __forceinline__ void epilogue_tma(uint32_t tmem, int quarter, int nco
 // segments, the rows of C it scales requested a piece ahead.  One lane per row,
 // as in store_tile, touches a cache line per lane: at 1537 x 2050 x 1100 that
 // and a separate alpha / beta pass took 28 of 90 us.
+template <bool SCALE>
 __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int ncols, int m0, int n0, int M, int N,
                                               float *__restrict__ C, int64_t ldc, float alpha, float beta, int ab,
                                               uint8_t *stage)
@@ -158,12 +159,12 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int nc
 #pragma unroll
         for (int r = 0; r < 32; ++r) next[r] = (c + lane < cols && r < nr) ? cp[(int64_t)r * ldc + c] : 0.0f;
     };
-    if (ab == 2) load_c(0);
+    if (SCALE && ab == 2) load_c(0);
 #pragma unroll 1
     for (int c = 0; c < cols; c += 32) {
         const bool mine = c + lane < cols;
         float old[32];
-        if (ab == 2) {
+        if (SCALE && ab == 2) {
 #pragma unroll
             for (int r = 0; r < 32; ++r) old[r] = next[r];
             load_c(c + 32);
@@ -174,12 +175,22 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int nc
 #pragma unroll
         for (int j = 0; j < 32; ++j) buf[lane * 33 + j] = __uint_as_float(v[j]);
         __syncwarp();
+        if constexpr (SCALE) {
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            float out = buf[r * 33 + lane];
-            if (ab != 0) out = __fmul_rn(alpha, out);
-            if (ab == 2) out = __fadd_rn(out, __fmul_rn(beta, old[r]));
-            if (mine && r < nr) cp[(int64_t)r * ldc + c] = out;
+            for (int r = 0; r < 32; ++r) {
+                float out = __fmul_rn(alpha, buf[r * 33 + lane]);
+                if (ab == 2) out = __fadd_rn(out, __fmul_rn(beta, old[r]));
+                if (mine && r < nr) cp[(int64_t)r * ldc + c] = out;
+            }
+        } else {
+            // the row pitch, hidden from the compiler, which would keep 32 multiples of it
+            // in registers
+            int64_t ld = ldc;
+            asm volatile("" : "+l"(ld));
+            float *p = cp + c;
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r, p += ld)
+                if (mine && r < nr) *p = buf[r * 33 + lane];
         }
         __syncwarp();
     }
@@ -190,8 +201,12 @@ __device__ __forceinline__ void epilogue_rows(uint32_t tmem, int quarter, int nc
 // to zero beforehand) instead of storing them.  c_tma: C is written through
 // the tensor map tmC.  pair_first >= 0 (BN = 128): CTA b computes quarter
 // b % 4 of 256 x 256 tile pair_first + b / 4 in the raster order of
-// prodsum_f32_pair_kernel, which ran the tiles before it.
-template <int BN, int KB, int STAGES, int SPLIT>
+// prodsum_f32_pair_kernel, which ran the tiles before it.  SCALE: ab is 1 or 2;
+// a kernel of its own, because the epilogue that reads C takes 247 registers (the
+// others 56), and CTAs with that many start later beside the last blocks of the
+// split: in one kernel 923 x 4 x 81 took 13.4 us, in two 12.6 (2048 x 1792 x 1 15.6 and
+// 15.0).
+template <int BN, int KB, int STAGES, int SPLIT, bool SCALE>
 __global__ void __launch_bounds__(192, 1)
 prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, int c_tma, int M, int N, int K, float *__restrict__ C,
@@ -226,7 +241,8 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
         mbar_init(accum_bar, 1);
-        for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
+        if (SCALE)
+            for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
         fence_mbar_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
@@ -263,11 +279,11 @@ prodsum_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         // ---------------- epilogue: TMEM -> registers -> C (tcgen05.ld needs the
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
-        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
+        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false, SCALE>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
                                                            cbar0 + 8u * (uint32_t)(warp & 3), flags);
         else if (ok && SPLIT == 1)
-            epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
-        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
+            epilogue_rows<SCALE>(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
+        else if (ok && nkb > 0 && c_tma) epilogue_tma<true, false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
                                                                    0, flags);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
@@ -311,7 +327,7 @@ struct F32PairCfg {
     static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 
-template <int BN, int KB, int STAGES, int SPLIT>
+template <int BN, int KB, int STAGES, int SPLIT, bool SCALE>
 __global__ void __launch_bounds__(192, 1)
 prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmC, int c_tma, int M, int N, int K,
@@ -339,7 +355,8 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
         mbar_init(accum_bar, 1);
-        for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
+        if (SCALE)
+            for (int w = 0; w < 4; ++w) mbar_init(cbar0 + 8u * w, 1);
         fence_mbar_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
@@ -399,11 +416,11 @@ prodsum_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // ---------------- epilogue of this CTA's 128 rows (tcgen05.ld needs the
         // whole warp, so a timeout in any lane skips the warp's epilogue)
         const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait(accum_bar, 0, flags));
-        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
+        if (ok && SPLIT == 1 && c_tma) epilogue_tma<false, SCALE>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, ab,
                                                            cbar0 + 8u * (uint32_t)(warp & 3), flags);
         else if (ok && SPLIT == 1)
-            epilogue_rows(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
-        else if (ok && nkb > 0 && c_tma) epilogue_tma<true>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
+            epilogue_rows<SCALE>(tmem, warp & 3, BN, m0, n0, M, N, C, ldc, alpha, beta, ab, base_ptr);
+        else if (ok && nkb > 0 && c_tma) epilogue_tma<true, false>(tmem, warp & 3, BN, m0, n0, M, N, &tmC, base, alpha, beta, 0,
                                                                    0, flags);
         else if (ok && nkb > 0) reduce_tile(tmem, warp & 3, 0, BN, m0, n0, M, N, C, ldc);
     }
@@ -438,7 +455,10 @@ cudaError_t run_f32(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, const u
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
     const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
-    auto kern = prodsum_f32_kernel<BN, KB, STAGES, SPLIT>;
+    auto kern = prodsum_f32_kernel<BN, KB, STAGES, SPLIT, false>;
+    if constexpr (SPLIT == 1) {
+        if (ab != 0) kern = prodsum_f32_kernel<BN, KB, STAGES, SPLIT, true>;
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t tiles = pair_first >= 0 ? 4 * pair_tiles : ((M + kBM - 1) / kBM) * ((N + BN - 1) / BN) * SPLIT;
@@ -474,7 +494,10 @@ cudaError_t run_f32_pair(int64_t M, int64_t N, int64_t K, const uint16_t *Ap, co
     static_assert(4 * BN * 128 <= STAGES * Cfg::STAGE, "TMA epilogue staging exceeds the stage memory");
     CUtensorMap tc = {};
     const int c_tma = make_c_map_f32(&tc, C, M, N, ldc) ? 1 : 0;
-    auto kern = prodsum_f32_pair_kernel<BN, KB, STAGES, SPLIT>;
+    auto kern = prodsum_f32_pair_kernel<BN, KB, STAGES, SPLIT, false>;
+    if constexpr (SPLIT == 1) {
+        if (ab != 0) kern = prodsum_f32_pair_kernel<BN, KB, STAGES, SPLIT, true>;
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t pairs = pair_tiles * SPLIT;
