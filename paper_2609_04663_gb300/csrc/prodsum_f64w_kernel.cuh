@@ -62,10 +62,11 @@
 // 2^(vA_i[row] + vB_j[col] - 16); columns' level exponents lie in shared
 // memory and each running sum is compared with its own element's bound.
 //
-// Warp roles: warp 0 lane 0 issues TMA loads (one 64-wide K-block of the A
-// slice and the B slice per stage), warp 1 owns TMEM and lane 0 issues the
-// MMAs (PAIR: the leader's), warps 4-19 drain and reduce.  Every wait is
-// bounded and reports EMU_FLAG_TIMEOUT instead of hanging.
+// Warp roles: warp 0 lane 0 issues TMA loads (64 of K of the A slice and the B
+// slice per stage, 128 on 128 x 128 tiles), warp 1 owns TMEM and an elected lane
+// of it issues the MMAs (PAIR: the leader's), warps 4-19 (4-11 on 256 columns)
+// drain and reduce.  Every wait is bounded and reports EMU_FLAG_TIMEOUT instead
+// of hanging.
 #pragma once
 
 #include "launchers.cuh"
@@ -91,8 +92,9 @@ struct F64WCfgT {
     // warpgroup 0: TMA producer (warp 0), MMA issuer + TMEM owner (warp 1), two
     // idle warps; then the drain warps: sixteen of BN / 4 columns each, or with
     // 256 columns eight of 128, whose threads have registers for their sums
-    // without spilling (sixteen threads' worth of addresses and temporaries
-    // beside 64 sums did not fit in 112 registers)
+    // (sixteen threads' worth of addresses and temporaries beside 64 sums did not
+    // fit in 112 registers).  Spills: none but in the row/column instances (74
+    // and 66 bytes at 256 columns, 16 at 256 x 128).
     static constexpr int FIRST_DRAIN = 4, DRAIN_WARPS = BN == 256 ? 8 : 16;
     static constexpr int DRAIN_THREADS = 32 * DRAIN_WARPS, THREADS = 128 + DRAIN_THREADS;
     static constexpr int COLS = BN / (DRAIN_WARPS / 4);                 // columns per drain thread
@@ -598,10 +600,13 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             // from the accumulator H (every earlier product is in it; this thread's own
             // reductions, so they precede the loads).  HC columns per chunk, from the third
             // chunk on, in time the warp would wait for partials, and the rest after the
-            // last chunk.  No branches in it: with a branch per element (a load for live rows only,
-            // the cases of the code) the loads were not in flight together and 128 columns took
-            // 64,000 clocks, now 20,000 (21 products of 16384 x 256 x 256: 298 -> 259 us, of
-            // 3000 x 3000 x 300: 440 -> 358).
+            // last chunk.  On pairs without branches: with a branch per element (a load
+            // for live rows only, the cases of the code) the loads were not in flight
+            // together and 128 columns took 64,000 clocks, now 20,000 (21 products of
+            // 16384 x 256 x 256: 298 -> 259 us, of 3000 x 3000 x 300: 440 -> 358).  Elsewhere
+            // every row is live, the loads stand together before the branches on the
+            // codes, and without those branches ptxas spreads them (128 x 30000 x 300: 283 ->
+            // 297 us).
             constexpr int HC = BN == 256 ? 16 : 8;
             auto code_columns = [&](int j0) {
                 double hd[HC];
@@ -621,8 +626,16 @@ prodsum_f64w_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         const uint32_t mh = xh & 0xFFFFFu;
                         const bool edge = ((n >= 0) & (mh == 0xFFFFFu)) | ((n > 0) & (mh == 0u)) | (n > kMaxRoundBits);
                         const uint32_t odd = ((uint32_t)__double2loint(h) & 1u) << 7;
-                        each |= edge;
-                        const uint32_t code = edge ? kCodeEach : n > 0 ? (uint32_t)(n + 48) | odd : kCodeKeep;
+                        uint32_t code = kCodeKeep;
+                        if constexpr (PAIR) {
+                            each |= edge;
+                            code = edge ? kCodeEach : n > 0 ? (uint32_t)(n + 48) | odd : kCodeKeep;
+                        } else if (edge) {
+                            code = kCodeEach;
+                            each = true;
+                        } else if (n > 0) {
+                            code = (uint32_t)(n + 48) | odd;
+                        }
                         cw |= code << (8 * k);
                     }
                     codes[(j0 / 4 + w) * Cfg::DRAIN_THREADS] = cw;
