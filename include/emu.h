@@ -152,8 +152,7 @@ emu_status emu_split_f64_slices(const double *X, int64_t rows, int64_t cols, int
 /* Workspace bytes for emu_gemm_f32 (mode 32) / emu_gemm_f64 (mode 64):
  * the flag word plus the slice planes of A (M x K) and B (K x N), and in
  * mode 64 the product-sum's FP64 accumulator (8 bytes per element of C,
- * rounded up to 128 x 128 tiles, or to 128 x 256 tiles where that is
- * larger). */
+ * rounded up to 128 x 256 tiles). */
 size_t emu_gemm_workspace_bytes(int mode, int64_t M, int64_t N, int64_t K);
 
 /* The split step of a GEMM C = A . B as one call: A (M x K, lda) into
@@ -161,8 +160,10 @@ size_t emu_gemm_workspace_bytes(int mode, int64_t M, int64_t N, int64_t K);
  * planes Bcomps [s][N][ldcomp] (ldcomp >= K), exactly as emu_split_f32 /
  * emu_split_f64_slices split each operand (planes and levels identical), in
  * fewer launches, as the GEMM entry points run it (FP32: one launch for
- * both; FP64: the level-0 maxima of both in one launch).  FP64: nslices in 3..6 as for emu_split_f64_slices; vA, vB:
- * device int32[6] receiving the level exponents of A and of B.  ws: at least
+ * both; FP64: one launch for small operands, else the level-0 maxima of both
+ * in one launch, a pass each and the verifier of both).  FP64: nslices in 3..6
+ * as for emu_split_f64_slices; vA, vB: device int32[6] receiving the level
+ * exponents of A and of B.  ws: at least
  * emu_split_workspace_bytes(mode); one flag word covers both operands.
  * Errors as the single-operand splits. */
 emu_status emu_split_f32_pair(int64_t M, int64_t N, int64_t K, const float *A, int64_t lda,
@@ -246,7 +247,7 @@ emu_status emu_gemm_f64_merged(int64_t M, int64_t N, int64_t K, const double *A,
  * without reading C; otherwise C = fl(fl(alpha * P) + fl(beta * C)).  K = 0
  * gives P = 0.  ws: device workspace of at least
  * emu_gemm_ex_workspace_bytes (the GEMM workspace plus an M x N product
- * buffer), 16-byte aligned.  Errors as emu_gemm_*; EMU_ERR_INVALID_ARG also
+ * buffer, which FP32 uses for K = 0 only), 16-byte aligned.  Errors as emu_gemm_*; EMU_ERR_INVALID_ARG also
  * for an op other than EMU_OP_N / EMU_OP_T. */
 #define EMU_OP_N 0
 #define EMU_OP_T 1

@@ -16,7 +16,7 @@ namespace {
 // formed by the same pair arithmetic as the split kernels, so C is
 // bit-identical to split + product-sum.
 //
-// Warp 0 owns TMEM and its lane 0 issues the MMAs.  CONV converter threads
+// Warp 0 owns TMEM and an elected lane issues the MMAs.  CONV converter threads
 // (warps 1 ..) load the FP32 tiles of A (128 x 32) and B (32 x 256) one K-block
 // ahead with coalesced loads, prefetch four K-blocks ahead into L2, split in
 // registers and store the slices into the stage in the 64-byte-swizzled

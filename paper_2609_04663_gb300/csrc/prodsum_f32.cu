@@ -8,7 +8,7 @@
 // slice serves all products that use it) into ONE FP32 accumulator in TMEM, in
 // the operand-reuse order of Eq. (fp32reuseorder).  The accumulator is read
 // once at the end.  Warp roles: warp 0 lane 0 issues TMA loads, warp 1 owns
-// TMEM and lane 0 issues the MMAs, warps 2-5 run the epilogue.  Every wait is
+// TMEM and an elected lane issues the MMAs, warps 2-5 run the epilogue.  Every wait is
 // bounded and reports EMU_FLAG_TIMEOUT instead of hanging.  The 128 x 256
 // plan runs on CTA pairs (prodsum_f32_pair_kernel: 256 x 256 tiles, the same
 // MMAs per output element).

@@ -1,7 +1,7 @@
 // Pieces shared by the FP32-mode product-sum kernels (the TMA-fed one and the
 // one that splits inside its producer): tile configuration, the MMA issue
-// loop of Eq. (fp32reuseorder) over a ring of stages (the epilogue is
-// store_tile of gemm_common.cuh).
+// loop of Eq. (fp32reuseorder) over a ring of stages.  The epilogues are in
+// prodsum_f32.cu; the one-kernel GEMM's is store_tile of gemm_common.cuh.
 #pragma once
 
 #include "gemm_common.cuh"

@@ -1,5 +1,5 @@
 // Tile shapes of the FP64-mode product-sum and the launches that cover a
-// result with them (the kernel is in prodsum_f64w.cu).
+// result with them (the kernel is in prodsum_f64w_kernel.cuh).
 #include <cstdlib>
 #include <cstring>
 
@@ -11,11 +11,12 @@ constexpr int kTileRows = 128;
 
 // Tile shape of the FP64 product-sum.  Every shape forms the same exact sums
 // and adds them with the same roundings, so C does not depend on the choice.
-// Per-SM rates relative to 256 x 256 tiles on CTA pairs (4096^3, 21 products,
-// every SM busy, 1446 TFLOP/s): 256 x 128 on pairs 0.82, 128 x 256 0.85, 128 x 128
-// 0.68, 128 x 64 0.39; a narrower tile moves more operand bytes through shared
-// memory per FLOP.  (A single wave of 256 x 128 tiles takes a little more than
-// the rate says: kRateHalf.)
+// The table below holds per-SM rates relative to 256 x 256 tiles on CTA pairs.
+// Measured at 4096^3 with 21 products, every SM busy (256 x 256: 1446 TFLOP/s), they
+// are 0.82 for 256 x 128 on pairs, 0.85, 0.68 and 0.39; a narrower tile moves more
+// operand bytes through shared memory per FLOP.  A single wave of 256 x 128 tiles takes
+// a little more than the rate says (kRateHalf), and the two narrowest are 0.66 and
+// 0.38 in the table, which leaves near ties to the wider tile.
 // - The shape with the least waves x columns / rate is taken.  Pairs need two
 //   128-row tile rows.
 // - 128 x 128 tiles are taken only where 256 x 128 pairs would leave half of the
